@@ -194,6 +194,10 @@ __global__ void __launch_bounds__(BATCH ? (WIDE ? 640 : 384) : (DEG >= 6 ? 640 :
     auto tAt = [&](uint32_t i) -> unsigned long long {
         if constexpr (BATCH) return __ldg(gT + i); else return sT[i];
     };
+    auto tHi = [&](uint32_t i) -> uint32_t {
+        if constexpr (BATCH) return __ldg(reinterpret_cast<const uint32_t *>(gT) + 2 * i + 1);
+        else return reinterpret_cast<const uint32_t *>(sT)[2 * i + 1];
+    };
     auto entries = [&](const uint4 &row, uint32_t *ent) {
         ent[0] = row.x & 0xFFFFu; ent[1] = row.x >> 16; ent[2] = row.y & 0xFFFFu; ent[3] = row.y >> 16;
         ent[4] = row.z & 0xFFFFu; ent[5] = row.z >> 16; ent[6] = row.w & 0xFFFFu; ent[7] = row.w >> 16;
@@ -597,8 +601,7 @@ __global__ void __launch_bounds__(BATCH ? (WIDE ? 640 : 384) : (DEG >= 6 ? 640 :
 #pragma unroll
             for (int l = 0; l < kRow; ++l)
                 if (real(l, ent)) cbase[ent[l] & 0x7FFFu] = static_cast<unsigned char>(cx[l] + delta);
-            const long long w = wpre(t);
-            ev += nX ? -w : w;
+            if (EXT) { const long long w = wpre(t); ev += nX ? -w : w; }
         }
         if (nY != yI) {
             ycol[q * 32] = yw ^ bit;
@@ -607,8 +610,19 @@ __global__ void __launch_bounds__(BATCH ? (WIDE ? 640 : 384) : (DEG >= 6 ? 640 :
 #pragma unroll
             for (int l = 0; l < kRow; ++l)
                 if (real(l, ent)) yb[ent[l] & 0x7FFFu] = static_cast<unsigned char>(cy[l] + delta);
-            const long long w = wpre(static_cast<long long>(t) - lag);
-            ev += nY ? w : -w;
+            if (EXT) { const long long w = wpre(static_cast<long long>(t) - lag); ev += nY ? w : -w; }
+        }
+        if (!EXT) {
+            // One lag: W(t) = a (a + 1) / 2 + (t - m) L with m = min(t, l), a = m - k + 1 (0 before
+            // k), and W(t - 1) = W(t) - a.  Two 32 x 32 -> 64-bit products for both chains' events.
+            const uint32_t m = min(t, ell);
+            if (m >= ws0) {
+                const uint32_t a = m - ws0 + 1u;
+                const long long w = static_cast<long long>((static_cast<unsigned long long>(a) * (a + 1u)) >> 1) +
+                                    static_cast<long long>(static_cast<unsigned long long>(t - m) * wcap);
+                if (nX != xI) ev += nX ? -w : w;
+                if (nY != yI) { const long long v = w - a; ev += nY ? v : -v; }
+            }
         }
         if (ev != 0) {
             red_add(racc(I), ev);
@@ -628,9 +642,13 @@ __global__ void __launch_bounds__(BATCH ? (WIDE ? 640 : 384) : (DEG >= 6 ? 640 :
         }
     };
 
-    // One step of the pair.  X's full conditional from its counts; when some lane of the warp
-    // has not met, Y's from its own column (a met lane reads its X column there, so Y = X).
-    // The uniform U = wu 2^32 + lo needs lo only when wu equals a threshold's high word.
+    // One step of the pair.  X's full conditional from its counts; a lane that has not met works
+    // Y's, from its own column, and both chains' flips in one branch of its own.  (Y worked by every
+    // lane of a warp that holds an unmet one, with a select per pool, measured 38.1 ms on 262,144
+    // slots of the low-noise 1298 x 97 design and 20.3 ms on 38,912 slots of a mixed-degree 2003 x
+    // 151 one; the branch 36.3 and 14.5 ms.)
+    // The uniform U = wu 2^32 + lo needs lo only when wu equals a threshold's high word, so a step
+    // loads the high word and a met lane leaves it after one compare unless the bit may flip.
     // The site a step word selects (alias draw).
     auto site_of = [&](uint32_t ws) -> uint32_t {
         const unsigned long long prod = static_cast<unsigned long long>(ws) * static_cast<uint32_t>(na);
@@ -656,80 +674,65 @@ __global__ void __launch_bounds__(BATCH ? (WIDE ? 640 : 384) : (DEG >= 6 ? 640 :
         }
         const uint32_t q = I >> 5, bit = 1u << (I & 31);
         const uint32_t xw = st[q * 32];
-        const uint32_t xI = (xw & bit) ? 1u : 0u;
+        const uint32_t xI = __funnelshift_r(xw, xw, I) & 1u;
         uint32_t ent[8];
         entries(row, ent);
-        uint32_t cx[kRow], cy[kRow];
-        uint32_t ix = 0;
+        // The index of the threshold table from the counts c of I's pools and I's own bit z: a pool
+        // decides when it holds no other positive (c - z = 0).
+        auto index = [&](const uint32_t *c, uint32_t z) -> uint32_t {
+            uint32_t ix = 0;
+#pragma unroll
+            for (int l = 0; l < kRow; ++l)
+                if (l < NE && (DEG > 0 || l < deg)) {
+                    if constexpr (MASKT) { if (c[l] == z) ix |= 1u << l; }
+                    else if (c[l] == z) ix += (ent[l] >> 15) ? 9u : 1u;
+                }
+            if constexpr (MASKT) ix += ent[kRow - 1] << 6;       // row of the positive-pool count
+            return ix;
+        };
+        uint32_t cx[kRow];
 #pragma unroll
         for (int l = 0; l < kRow; ++l) {
             cx[l] = 0u;
-            cy[l] = 0u;
-            if (l < NE && (DEG > 0 || l < deg)) {
-                if constexpr (MASKT) {     // plain offsets, positive-outcome pools first
-                    cx[l] = cbase[ent[l]];
-                    if (cx[l] == xI) ix |= 1u << l;                // c_j - x_I = 0: pool j decides
-                } else {
-                    cx[l] = cbase[ent[l] & 0x7FFFu];
-                    if (cx[l] == xI) ix += (ent[l] >> 15) ? 9u : 1u;
-                }
-            }
+            if (l < NE && (DEG > 0 || l < deg)) cx[l] = cbase[MASKT ? ent[l] : ent[l] & 0x7FFFu];
         }
-        if constexpr (MASKT) ix += ent[kRow - 1] << 6;           // row of the positive-pool count
-        const unsigned long long TX = tAt(ix);
-        unsigned long long TY = TX;
-        uint32_t yw = xw, yI = xI;
-        bool own = false;
-        // Y's side, for the lanes that have not met (a met lane keeps Y = X).
-        auto ypart = [&](const uint32_t *yp) {
-            const unsigned char *yb = reinterpret_cast<const unsigned char *>(yp);
-            yw = own ? yp[q * 32] : xw;
-            yI = (yw & bit) ? 1u : 0u;
-            uint32_t iy = 0;
+        const uint32_t ix = index(cx, xI);
+        const uint32_t thx = tHi(ix);
+        // The new bit of a chain whose threshold (entry i) has the high word th.
+        auto decide = [&](uint32_t th, uint32_t i) -> uint32_t {
+            uint32_t nb = wu < th ? 1u : 0u;
+            if (wu == th) {
+                const uint32_t lo = philox_low_word(make_uint4(t, r, slot_g, instance | (2u << 24)), k0, k1);
+                nb = lo < static_cast<uint32_t>(tAt(i)) ? 1u : 0u;
+            }
+            return nb;
+        };
+        auto trace_step = [&](uint32_t xf, uint32_t yf) {
+            if constexpr (TRACE) {
+                // draw t moves X_{t+1} and, from t = L on, Y_{t+1-L}; a pair that has met moves both
+                // alike, and before t = L Y stays at Y_0
+                if (trec && t < static_cast<uint32_t>(p.trace_steps))
+                    trec[4 + t] = static_cast<int32_t>(I | (xf << 16) | (yf << 17));
+            }
+        };
+        if (COUPLED && D != 0) {
+            const unsigned char *yb = reinterpret_cast<const unsigned char *>(ycol);
+            const uint32_t yw = ycol[q * 32];
+            const uint32_t yI = __funnelshift_r(yw, yw, I) & 1u;
+            uint32_t cy[kRow];
 #pragma unroll
             for (int l = 0; l < kRow; ++l) {
-                if (l < NE && (DEG > 0 || l < deg)) {
-                    if constexpr (MASKT) {
-                        cy[l] = own ? static_cast<uint32_t>(yb[ent[l]]) : cx[l];
-                        if (cy[l] == yI) iy |= 1u << l;
-                    } else {
-                        cy[l] = own ? static_cast<uint32_t>(yb[ent[l] & 0x7FFFu]) : cx[l];
-                        if (cy[l] == yI) iy += (ent[l] >> 15) ? 9u : 1u;
-                    }
-                }
+                cy[l] = 0u;
+                if (l < NE && (DEG > 0 || l < deg)) cy[l] = yb[MASKT ? ent[l] : ent[l] & 0x7FFFu];
             }
-            if constexpr (MASKT) iy += ent[kRow - 1] << 6;
-            TY = tAt(iy);
-        };
-        if (COUPLED) {
-            const bool ymode = __any_sync(__activemask(), D != 0);
-            if (ymode) {
-                own = D != 0;
-                ypart(ycol);
-            }
-        }
-        const uint32_t thx = static_cast<uint32_t>(TX >> 32), thy = static_cast<uint32_t>(TY >> 32);
-        uint32_t nX = wu < thx ? 1u : 0u, nY = wu < thy ? 1u : 0u;
-        if (wu == thx || wu == thy) {
-            const uint32_t lo = philox_low_word(make_uint4(t, r, slot_g, instance | (2u << 24)), k0, k1);
-            if (wu == thx) nX = lo < static_cast<uint32_t>(TX) ? 1u : 0u;
-            if (wu == thy) nY = lo < static_cast<uint32_t>(TY) ? 1u : 0u;
-        }
-        if constexpr (TRACE) {
-            // draw t moves X_{t+1} and, from t = L on, Y_{t+1-L}; a pair that has met moves both
-            // alike, and before t = L Y stays at Y_0
-            if (trec && t < static_cast<uint32_t>(p.trace_steps)) {
-                const uint32_t xf = nX != xI ? 1u : 0u;
-                const uint32_t yf = !COUPLED ? 0u
-                                    : own ? ((nY != yI && !(EXT && t < v_lag())) ? 1u : 0u)
-                                          : (xf && t >= v_lag() ? 1u : 0u);
-                trec[4 + t] = static_cast<int32_t>(I | (xf << 16) | (yf << 17));
-            }
-        }
-        if (COUPLED && own) {
+            const uint32_t iy = index(cy, yI);
+            const uint32_t nX = decide(thx, ix), nY = decide(tHi(iy), iy);
+            trace_step(nX ^ xI, ((nY != yI) && !(EXT && t < v_lag())) ? 1u : 0u);
             if ((nX ^ xI) | (nY ^ yI)) unmet_flip(I, q, bit, xw, yw, xI, yI, nX, nY, ent, cx, cy);
-        } else if (nX != xI) {
-            met_flip(I, q, bit, xw, nX, ent, cx);
+        } else if (TRACE || (xI ? wu >= thx : wu <= thx)) {
+            const uint32_t nX = decide(thx, ix);
+            trace_step(nX ^ xI, COUPLED && nX != xI && t >= v_lag() ? 1u : 0u);
+            if (nX != xI) met_flip(I, q, bit, xw, nX, ent, cx);
         }
         ++t;
         if (SYSTEMATIC) { ++sysI; if (sysI == static_cast<uint32_t>(na)) sysI = 0; }
