@@ -69,8 +69,8 @@ typedef struct mcpd_params {
     int32_t scan;              /* MCPD_SCAN_*                                                     */
     int32_t coupled;           /* 1: Algorithms 3-4 (coupled pairs, unbiased); 0: Algorithms 1-2
                                   (one chain per replication, burn-in average)                    */
-    int32_t lanes_per_pair;    /* 0: automatic; 1: one thread per pair (the only layout of this
-                                  build)                                                          */
+    int32_t lanes_per_pair;    /* 0: automatic; 1: the sampling kernel (the only layout of a single
+                                  instance in this build)                                         */
     const double *scan_weights;   /* MCPD_SCAN_CUSTOM: [n_active] positive weights, host          */
     const double *init_marginals; /* NULL: Z_0 = 0 (all negative); else [n_active] in [0,1], host:
                                   Z_0 ~ prod_i Bernoulli(nu_i)                                    */
@@ -113,8 +113,8 @@ typedef struct mcpd_params {
     int64_t trace_reps;        /* replications recorded per traced slot (0: 8); at most 1024      */
 } mcpd_params;
 
-/* Counters of one run.  site_updates, reps_started, reps_retained and tau_over_audit are -1 if a
- * pair ran 2^32 or more progress units in one launch (this build keeps them in 32-bit halves). */
+/* Counters of one run.  progress_units and site_updates count the method's draws and updates (a
+ * pair's, to the end of its replication), not the steps the kernel takes for them. */
 typedef struct mcpd_stats {
     int64_t progress_units;    /* shared draws executed, aborted replications included            */
     int64_t site_updates;      /* single-site updates executed (2 per coupled draw but the L
@@ -127,8 +127,8 @@ typedef struct mcpd_stats {
     int64_t n_active;
     double kernel_ms;          /* device time of the sampling kernel (CUDA events)                */
     int64_t tau_over_audit;    /* completed replications with tau > params.tau_audit             */
-    int64_t resident_pairs;    /* pairs the sampling kernel held at once (grid x block; the widest
-                                  size class of a batch)                                         */
+    int64_t resident_pairs;    /* slots the sampling kernel works on at once (its warps x the slots
+                                  of a chunk, at most 32; the widest class of a batch)           */
     int64_t h2d_bytes, d2h_bytes; /* single instance: bytes the library copied host -> device and
                                   device -> host for this plan so far (tables at creation; counters
                                   at each collect; fetches; mcpd_decode adds its est/se copies);
@@ -157,7 +157,7 @@ void mcpd_plan_destroy(mcpd_plan *plan);
 
 /* Plan facts: info[0] n_active, [1] n_buckets, [2] horizon B, [3] k (burn b uncoupled),
  * [4] l (b + T - 1 uncoupled), [5] L (window length), [6] slots P, [7] warps per block,
- * [8] resident pairs, [9] shared-memory bytes per block, [10] lanes per pair. */
+ * [8] lanes of the launch (32 per warp), [9] shared-memory bytes per block, [10] 1. */
 int mcpd_plan_info(const mcpd_plan *plan, int64_t info[16]);
 /* active[a] = original index of the a-th retained clone (ascending). */
 int mcpd_plan_active(const mcpd_plan *plan, int32_t *active);
@@ -175,8 +175,8 @@ int mcpd_run_async(mcpd_ctx *ctx, mcpd_plan *plan, double *est_dev, double *se_d
  * receive theta_CT and its standard error over all S + slots slots (Theorem 2: the slot means are
  * i.i.d., so the estimator over more slots is the same estimator with a larger P).  Every slot
  * keeps the plan's horizon B, so the result is bit-identical to one mcpd_run_async of a plan with
- * P = S + slots and horizon B.  The launch keeps the plan's grid with its warps per block trimmed
- * to whole rounds of these slots.  S + slots <= 2^31 and slot_offset + S + slots <= 2^32;
+ * P = S + slots and horizon B.  The launch keeps the plan's grid, with warps per block (at most the
+ * plan's) and slots per warp fitted to these slots.  S + slots <= 2^31 and slot_offset + S + slots <= 2^32;
  * per-slot records and traces (record_slots, trace_stride) allow only accumulate = 0 with
  * slots <= the plan's P.  Asynchronous; mcpd_collect reads this run's counters and kernel time. */
 int mcpd_run_slots_async(mcpd_ctx *ctx, mcpd_plan *plan, int64_t slots, int32_t accumulate,
@@ -259,15 +259,15 @@ int mcpd_batch_classes(int32_t n_inst, const mcpd_design *designs, const uint8_t
 /* info[0] total retained clones, [1] instances, [2] total slots, [3] largest n_active,
  * [4] warps per block, [5] blocks and [7] shared-memory bytes per block of the first class (the
  * largest pair state of its degree group), [6] resident pairs of the widest class, [8] lanes
- * per pair, [9] size
- * classes, [10] largest warps per block over the classes, [11] classes that launch the kernel
- * variant with meeting caps and lags > 1, [12] classes that launch a build with a compile-time
+ * per pair (1: the sampling kernel), [9] size
+ * classes, [10] largest warps per block over the classes, [11] classes
+ * with meeting caps or lags > 1, [12] classes that launch a build with a compile-time
  * degree (coupled classes whose instances all sit in the same number of pools per clone, 3 to 8;
  * thresholds indexed by the mask of deciding pools up to 6). */
 int mcpd_batch_info(const mcpd_batch *batch, int64_t info[16]);
 /* offsets: [n_inst + 1] host array receiving each instance's first output index. */
 int mcpd_batch_offsets(const mcpd_batch *batch, int64_t *offsets);
-/* Choose the launch shape of every class: lanes per pair (1: one thread per pair; 8, 16 or 32: a
+/* Choose the launch shape of every class: lanes per pair (1: the sampling kernel; 8, 16 or 32: a
  * lane group per pair, coupled batches only; all give identical results) and at most
  * warps_per_block warps per block (0: as many as the kernel and the class's largest pair state
  * allow).  May reallocate the per-pair scratch; invalidates a captured graph. */

@@ -46,6 +46,9 @@ struct mcpd_plan {
     int64_t slots_run = 0;           // slots in the buckets since the last run that cleared them
     long long last_pairs = 0;        // pairs the last launch held (its grid x block)
     mutable int64_t h2d_bytes = 0, d2h_bytes = 0;   // bytes copied between host and device (fetches too)
+    size_t scratch_words() const {
+        return static_cast<size_t>(grid) * (block / 32) * mcpd::warp_words(kp.bank, t.na);
+    }
 };
 
 namespace {
@@ -203,8 +206,7 @@ int mcpd_plan_create(mcpd_ctx *ctx, const mcpd_design *design, const uint8_t *y,
     const mcpd::Tables &t = pl->t;
     if (cudaSetDevice(ctx->device) != cudaSuccess) { delete pl; return set_err(ctx, MCPD_ECUDA, "cudaSetDevice"); }
 
-    // Launch shape: tables first in shared memory, then one 32-column region per warp and the
-    // Y regions.
+    // Launch shape: tables first in shared memory, then one 32-column region per warp.
     const size_t tables = mcpd::kernel_table_bytes(t);
     mcpd::PairsShape shape;
     rc = mcpd::pairs_shape(t.coupled, t.scan, t.udeg, false, tables, t.wpp, ctx->smem_optin, t.P,
@@ -234,8 +236,12 @@ int mcpd_plan_create(mcpd_ctx *ctx, const mcpd_design *design, const uint8_t *y,
     ALLOC(d_T, mcpd::kernel_T(t).size());
     ALLOC(d_Tnu, t.Tnu.size());
     ALLOC(d_init, t.init_pairs.size());
-    ALLOC(kp.pair_scratch, static_cast<size_t>(pl->pairs) * mcpd::pair_words(t.na, t.W));
-    ALLOC(kp.y_state, static_cast<size_t>(pl->pairs) * t.wpp);
+    {
+        const mcpd::ChunkShape cs = mcpd::chunk_shape(t.P, pl->grid, warps, 32 * mcpd::kBankRounds);
+        kp.chunk = cs.chunk;
+        kp.bank = std::max(32, cs.chunk);         // a later run may bring more slots
+    }
+    ALLOC(kp.pair_scratch, pl->scratch_words());
     ALLOC(kp.S1, static_cast<size_t>(t.nb) * t.na);
     ALLOC(kp.S2lo, static_cast<size_t>(t.nb) * t.na);
     ALLOC(kp.S2hi, static_cast<size_t>(t.nb) * t.na);
@@ -280,7 +286,6 @@ int mcpd_plan_create(mcpd_ctx *ctx, const mcpd_design *design, const uint8_t *y,
     kp.seed = t.seed; mcpd::philox_round_keys(t.seed, kp.rk); kp.instance = t.instance; kp.warps = warps;
     kp.smem_tables = static_cast<uint32_t>(tables);
     kp.nT = static_cast<int32_t>(mcpd::kernel_T(t).size());
-    kp.y_regions = shape.y_regions;
     CU_OR(cudaEventCreate(&pl->ev0), mcpd_plan_destroy(pl));
     CU_OR(cudaEventCreate(&pl->ev1), mcpd_plan_destroy(pl));
     CU_OR(cudaStreamSynchronize(ctx->stream), mcpd_plan_destroy(pl));
@@ -325,18 +330,14 @@ int run_range(mcpd_ctx *ctx, mcpd_plan *pl, int64_t slots, bool accumulate, doub
     mcpd::KParams kp = pl->kp;
     kp.P = slots;
     kp.slot_offset = t.slot_offset + first;
-    // Launch shape: the plan's, with its warps per block trimmed to the fewest that need no more
-    // rounds of slots for this run (the plan's own slot count gives the plan's shape).
-    int warps = pl->block / 32;
-    {
-        const long long per_round = static_cast<long long>(pl->grid) * 32;
-        const long long rounds = (slots + per_round * warps - 1) / (per_round * warps);
-        const long long w = (slots + rounds * per_round - 1) / (rounds * per_round);
-        if (w >= 1 && w < warps) warps = static_cast<int>(w);
-    }
+    // Launch shape: the plan's grid, with the warps per block (at most the plan's) and the chunk for
+    // this run's slots (the plan's own slot count gives the plan's shape).
+    const mcpd::ChunkShape cs = mcpd::chunk_shape(slots, pl->grid, pl->block / 32, kp.bank);
+    const int warps = cs.warps;
+    const long long all_warps = static_cast<long long>(pl->grid) * warps;
     kp.warps = warps;
-    kp.y_regions = mcpd::pairs_y_regions(t.coupled, warps);
-    const size_t smem = mcpd::pairs_smem_bytes(kp.smem_tables, t.wpp, warps, kp.y_regions);
+    kp.chunk = cs.chunk;
+    const size_t smem = mcpd::pairs_smem_bytes(kp.smem_tables, t.wpp, warps);
     const size_t nbna = static_cast<size_t>(t.nb) * t.na;
     if (!accumulate) {
         CU(cudaMemsetAsync(kp.S1, 0, nbna * 8, ctx->stream));
@@ -347,8 +348,7 @@ int run_range(mcpd_ctx *ctx, mcpd_plan *pl, int64_t slots, bool accumulate, doub
     CU(cudaMemsetAsync(kp.counters, 0, mcpd::kNumCounters * 8, ctx->stream));
     CU(cudaMemsetAsync(kp.error, 0, sizeof(int), ctx->stream));
     if (pl->dirty) {   // the kernel leaves these zeroed when it completes normally
-        CU(cudaMemsetAsync(kp.pair_scratch, 0, static_cast<size_t>(pl->pairs) * mcpd::pair_words(t.na, t.W) * 8, ctx->stream));
-        CU(cudaMemsetAsync(kp.y_state, 0, static_cast<size_t>(pl->pairs) * t.wpp * 4, ctx->stream));
+        CU(cudaMemsetAsync(kp.pair_scratch, 0, pl->scratch_words() * 8, ctx->stream));
     }
     if (kp.trace_G) CU(cudaMemsetAsync(kp.trace_G, 0, static_cast<size_t>(pl->n_trace) * t.na * 8, ctx->stream));
     if (kp.trace_rec)
@@ -370,7 +370,7 @@ int run_range(mcpd_ctx *ctx, mcpd_plan *pl, int64_t slots, bool accumulate, doub
         return set_err(ctx, MCPD_ECUDA, "finalize kernel launch");
     pl->ran = true;
     pl->slots_run = first + slots;
-    pl->last_pairs = static_cast<long long>(pl->grid) * warps * 32;
+    pl->last_pairs = all_warps * std::min(32, kp.chunk);
     return MCPD_OK;
 }
 
@@ -548,8 +548,9 @@ struct BatchClass {
     mcpd::BParams bp{};                // this class's launch arguments (insts = d_insts + first)
     int grid = 0, block = 0, warps = 0;
     size_t smem = 0;
-    long long pairs = 0, scratch_pairs = 0;
-    std::vector<void *> scratch;       // per-pair scratch (resized by the tuner)
+    long long pairs = 0;
+    size_t scratch_words = 0, scratch_held = 0;   // in use by the shape; allocated
+    std::vector<void *> scratch;       // sampling scratch (resized by the tuner)
 };
 
 struct mcpd_batch {
@@ -605,15 +606,32 @@ void free_list(std::vector<void *> &list) {
     list.clear();
 }
 
-// Launch shape of every class: `lanes` per pair (1: one thread per pair; 8, 16, 32: a lane group
+// Number each class's chunks (slots of one instance, at most its bank) in the descriptors `insts`.
+void number_units(mcpd_batch *b, std::vector<mcpd::InstDesc> &insts) {
+    for (BatchClass &c : b->cls) {
+        long long at = 0;
+        for (int32_t k = 0; k < c.count; ++k) {
+            mcpd::InstDesc &d = insts[static_cast<size_t>(c.first) + k];
+            d.unit_begin = at;
+            d.units = c.bp.bank > 0 ? (d.P + c.bp.bank - 1) / c.bp.bank : 0;
+            at += d.units;
+        }
+        c.bp.total_units = at;
+    }
+}
+
+// Launch shape of every class: `lanes` per pair (1: the sampling kernel; 8, 16, 32: a lane group
 // per pair) and at most `warps` per block (0: as many as fit the class's largest pair state),
-// and the per-pair scratch it needs.
+// the chunks, and the scratch it needs.
 int batch_shape(mcpd_ctx *ctx, mcpd_batch *b, int warps, int lanes = 1) {
     if (lanes != 1 && lanes != 8 && lanes != 16 && lanes != 32)
         return set_err(ctx, MCPD_EINVAL, "lanes per pair must be 1, 8, 16 or 32");
     if (lanes > 1 && !b->coupled) return set_err(ctx, MCPD_EINVAL, "lane groups run coupled batches only");
+    double work = 0.0;                 // columns x words of all classes: what they share the GPU by
+    for (const BatchClass &c : b->cls) work += static_cast<double>(b->total_work0[&c - b->cls.data()]) * c.bp.max_wpp;
     for (size_t ci = 0; ci < b->cls.size(); ++ci) {
         BatchClass &c = b->cls[ci];
+        const long long class_slots = b->total_work0[ci];
         int per_sm = 1, w = 0;
         if (lanes == 1) {
             mcpd::PairsShape shape;
@@ -628,9 +646,22 @@ int batch_shape(mcpd_ctx *ctx, mcpd_batch *b, int warps, int lanes = 1) {
             }
             w = shape.warps;
             c.smem = shape.smem;
-            c.bp.y_regions = shape.y_regions;
-            c.bp.wide = shape.wide ? 1 : 0;
             per_sm = shape.per_sm;
+            // The class's part of the GPU's warps, and the slots that makes for each.
+            const long long resident = static_cast<long long>(ctx->sm_count) * per_sm * w;
+            const double part = work > 0 ? static_cast<double>(class_slots) * c.bp.max_wpp / work : 1.0;
+            c.bp.bank = static_cast<int32_t>(std::max<long long>(1, std::min<long long>(32, static_cast<long long>(
+                class_slots / std::max(1.0, resident * part)) + 1)));
+            long long units = 0;
+            for (int32_t k = 0; k < c.count; ++k)
+                units += (b->insts0[static_cast<size_t>(c.first) + k].P + c.bp.bank - 1) / c.bp.bank;
+            // A class with fewer chunks than resident warps launches only the blocks they fill: a
+            // block keeps its shared memory until its last warp ends, so blocks whose warps find
+            // no chunk would hold SMs that the concurrently running classes need.
+            c.grid = static_cast<int>(std::max<long long>(1, std::min<long long>(static_cast<long long>(ctx->sm_count) * per_sm,
+                                                                                  (units + w - 1) / w)));
+            c.pairs = static_cast<long long>(c.grid) * w * std::min(32, c.bp.bank);
+            c.scratch_words = static_cast<size_t>(c.grid) * w * mcpd::warp_words(c.bp.bank, c.bp.max_na);
         } else {
             const size_t per_warp = static_cast<size_t>(32 / lanes) * 2 * c.bp.max_wpp * 4;
             const int cap = mcpd::group_max_threads(lanes) / 32;
@@ -638,34 +669,35 @@ int batch_shape(mcpd_ctx *ctx, mcpd_batch *b, int warps, int lanes = 1) {
             if (fit < 1) return set_err(ctx, MCPD_ETOO_LARGE, "largest instance does not fit one warp of pair state");
             w = warps > 0 ? std::min(warps, fit) : fit;
             c.smem = per_warp * w;
-            c.bp.y_regions = 0;
             // a permission shared by the launches of all classes: the device's opt-in maximum
             if (mcpd::set_group_smem(lanes, ctx->smem_optin) != MCPD_OK) return set_err(ctx, MCPD_ECUDA, "cudaFuncSetAttribute");
             if (mcpd::group_occupancy(lanes, w * 32, c.smem, &per_sm) != MCPD_OK || per_sm < 1) per_sm = 1;
+            // only the blocks the class's slots fill, as above
+            const long long pairs_per_block = std::max(1, w * 32 / lanes);
+            c.grid = static_cast<int>(std::max<long long>(
+                1, std::min<long long>(static_cast<long long>(ctx->sm_count) * per_sm,
+                                       (class_slots + pairs_per_block - 1) / pairs_per_block)));
+            c.pairs = static_cast<long long>(c.grid) * w * 32 / lanes;
+            c.scratch_words = static_cast<size_t>(c.pairs) * mcpd::pair_words(c.bp.max_na, c.bp.max_W);
         }
         c.warps = w;
         c.block = w * 32;
         c.bp.lanes = lanes;
-        // A class with fewer slots than one full launch holds pairs for launches only the blocks
-        // its slots fill: a block keeps its shared memory until its last warp ends, so blocks
-        // whose warps find no slot would hold SMs that the concurrently running classes need.
-        const long long class_slots = ci < b->total_work0.size() ? b->total_work0[ci] : c.bp.total_work;
-        const long long pairs_per_block = std::max(1, c.block / lanes);
-        c.grid = static_cast<int>(std::max<long long>(
-            1, std::min<long long>(static_cast<long long>(ctx->sm_count) * per_sm,
-                                   (class_slots + pairs_per_block - 1) / pairs_per_block)));
-        c.pairs = static_cast<long long>(c.grid) * c.block / lanes;
-        if (c.pairs > c.scratch_pairs) {
+        if (c.scratch_words > c.scratch_held) {
             free_list(c.scratch);
-            int rc;
-            if ((rc = balloc(ctx, c.scratch, &c.bp.pair_scratch,
-                             static_cast<size_t>(c.pairs) * mcpd::pair_words(c.bp.max_na, c.bp.max_W))) != MCPD_OK)
-                return rc;
-            if ((rc = balloc(ctx, c.scratch, &c.bp.y_state, static_cast<size_t>(c.pairs) * c.bp.max_wpp)) != MCPD_OK) return rc;
-            c.scratch_pairs = c.pairs;
-            b->dirty = true;
+            c.scratch_held = 0;
+            const int rc = balloc(ctx, c.scratch, &c.bp.pair_scratch, c.scratch_words);
+            if (rc != MCPD_OK) return rc;
+            c.scratch_held = c.scratch_words;
         }
     }
+    // The kernels lay the scratch out by their shape, so a run in another shape starts from a
+    // cleared one; the chunks are the descriptors' too.
+    b->dirty = true;
+    number_units(b, b->insts0);
+    number_units(b, b->insts);
+    CU(cudaMemcpyAsync(b->d_insts, b->insts.data(), sizeof(mcpd::InstDesc) * b->insts.size(), cudaMemcpyHostToDevice,
+                       ctx->stream));
     b->lanes = lanes;
     if (b->graph_exec) { cudaGraphExecDestroy(b->graph_exec); b->graph_exec = nullptr; }
     if (b->graph) { cudaGraphDestroy(b->graph); b->graph = nullptr; }
@@ -677,6 +709,7 @@ int restore_descriptors(mcpd_ctx *ctx, mcpd_batch *b) {
     if (!b->extended) return MCPD_OK;
     b->insts = b->insts0;
     for (size_t c = 0; c < b->cls.size(); ++c) b->cls[c].bp.total_work = b->total_work0[c];
+    number_units(b, b->insts);
     CU(cudaMemcpyAsync(b->d_insts, b->insts.data(), sizeof(mcpd::InstDesc) * b->insts.size(), cudaMemcpyHostToDevice,
                        ctx->stream));
     b->extended = false;
@@ -694,9 +727,7 @@ int batch_enqueue(mcpd_ctx *ctx, mcpd_batch *b, double *est_dev, double *se_dev,
     CU(cudaMemsetAsync(b->d_error, 0, sizeof(int), s));
     for (BatchClass &c : b->cls) {
         if (b->dirty || always_clear) {
-            CU(cudaMemsetAsync(c.bp.pair_scratch, 0,
-                               static_cast<size_t>(c.pairs) * mcpd::pair_words(c.bp.max_na, c.bp.max_W) * 8, s));
-            CU(cudaMemsetAsync(c.bp.y_state, 0, static_cast<size_t>(c.pairs) * c.bp.max_wpp * 4, s));
+            CU(cudaMemsetAsync(c.bp.pair_scratch, 0, c.scratch_words * 8, s));
         }
     }
     CU(cudaEventRecord(b->fork, s));
@@ -856,7 +887,6 @@ int mcpd_batch_create(mcpd_ctx *ctx, int32_t n_inst, const mcpd_design *designs,
         mcpd::BParams &bp = c.bp;
         bp.total_work = work;
         if (t.capped || t.lag > 1) bp.ext = 1;
-        if (!t.Tnu.empty()) bp.any_init = 1;
         // the class's uniform degree: the first instance's, kept while every instance shares it
         if (d.work_begin == 0) bp.udeg = t.udeg;
         else if (bp.udeg != t.udeg) bp.udeg = 0;
@@ -973,6 +1003,7 @@ int mcpd_batch_extend_async(mcpd_ctx *ctx, mcpd_batch *b, const int32_t *mask, d
         }
         c.bp.total_work = work;
     }
+    number_units(b, b->insts);
     b->extended = true;
     CU(cudaMemcpyAsync(b->d_insts, b->insts.data(), sizeof(mcpd::InstDesc) * b->insts.size(), cudaMemcpyHostToDevice,
                        ctx->stream));

@@ -6,12 +6,12 @@
 
 namespace mcpd {
 
-PairsKernelFn pick_batch_degree(int udeg, bool wide) {
+PairsKernelFn pick_batch_degree(int udeg) {
     switch (udeg) {
-        case 4: return wide ? pairs_kernel<true, false, true, 4, true> : pairs_kernel<true, false, true, 4, false>;
-        case 5: return wide ? pairs_kernel<true, false, true, 5, true> : pairs_kernel<true, false, true, 5, false>;
-        case 7: return wide ? pairs_kernel<true, false, true, 7, true> : pairs_kernel<true, false, true, 7, false>;
-        case 8: return wide ? pairs_kernel<true, false, true, 8, true> : pairs_kernel<true, false, true, 8, false>;
+        case 4: return pairs_kernel<true, false, true, 4>;
+        case 5: return pairs_kernel<true, false, true, 5>;
+        case 7: return pairs_kernel<true, false, true, 7>;
+        case 8: return pairs_kernel<true, false, true, 8>;
         default: return nullptr;
     }
 }

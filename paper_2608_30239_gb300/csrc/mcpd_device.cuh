@@ -29,6 +29,29 @@ static __device__ __forceinline__ uint4 philox10_rk(uint4 c, const uint32_t (&rk
     return c;
 }
 
+constexpr uint32_t kPhiloxM0 = 0xD2511F53u, kPhiloxM1 = 0xCD9E8D57u, kPhiloxW0 = 0x9E3779B9u, kPhiloxW1 = 0xBB67AE85u;
+
+// Rounds 3 to 10 on the state after two rounds: with the third round's keys, or the key table above.
+static __device__ __forceinline__ uint4 philox_tail(uint4 c, uint32_t k0, uint32_t k1) {
+#pragma unroll
+    for (int round = 2; round < 10; ++round) {
+        if (round > 2) { k0 += kPhiloxW0; k1 += kPhiloxW1; }
+        const uint32_t hi0 = __umulhi(kPhiloxM0, c.x), lo0 = kPhiloxM0 * c.x;
+        const uint32_t hi1 = __umulhi(kPhiloxM1, c.z), lo1 = kPhiloxM1 * c.z;
+        c = make_uint4(hi1 ^ c.y ^ k0, lo1, hi0 ^ c.w ^ k1, lo0);
+    }
+    return c;
+}
+static __device__ __forceinline__ uint4 philox_tail_rk(uint4 c, const uint32_t (&rk)[20]) {
+#pragma unroll
+    for (int round = 2; round < 10; ++round) {
+        const uint32_t hi0 = __umulhi(kPhiloxM0, c.x), lo0 = kPhiloxM0 * c.x;
+        const uint32_t hi1 = __umulhi(kPhiloxM1, c.z), lo1 = kPhiloxM1 * c.z;
+        c = make_uint4(hi1 ^ c.y ^ rk[2 * round], lo1, hi0 ^ c.w ^ rk[2 * round + 1], lo0);
+    }
+    return c;
+}
+
 // Word 0 of a block, out of line (the rare draw of a uniform's low half).
 static __device__ __noinline__ uint32_t philox_low_word(uint4 c, uint32_t k0, uint32_t k1) {
     return philox10(c, k0, k1).x;
@@ -41,8 +64,17 @@ static __device__ __forceinline__ void red_add(long long *a, long long v) {
 static __device__ __forceinline__ void red_max(unsigned long long *a, unsigned long long v) {
     asm volatile("red.global.max.u64 [%0], %1;" ::"l"(a), "l"(v) : "memory");
 }
-static __device__ __forceinline__ void red_or(uint32_t *a, uint32_t v) {
-    asm volatile("red.global.or.b32 [%0], %1;" ::"l"(a), "r"(v) : "memory");
+// W(u) for any lag: sum_{r=k}^{min(l,u)} (floor((u - r) / lag) + 1), through
+// F(n) = sum_{d=0}^{n} floor(d / lag) = lag q (q - 1) / 2 + q (n - q lag + 1), q = floor(n / lag).
+static __device__ __noinline__ long long lag_prefix(long long u, long long k, long long ell, long long lag) {
+    if (u < k) return 0;
+    const long long m = u < ell ? u : ell;
+    auto F = [&](long long n) -> long long {
+        if (n < 0) return 0;
+        const long long q = n / lag;
+        return lag * q * (q - 1) / 2 + q * (n - q * lag + 1);
+    };
+    return (m - k + 1) + F(u - k) - F(u - m - 1);
 }
 
 // Add G and G^2 (128-bit, carried into the high word) of one slot to bucket N*_p - 1.

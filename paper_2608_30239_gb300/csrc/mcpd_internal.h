@@ -2,6 +2,7 @@
 #pragma once
 #include <stdint.h>
 
+#include <algorithm>
 #include <string>
 #include <vector>
 
@@ -24,7 +25,7 @@ namespace mcpd {
 constexpr int kRow = 8;              // pool entries per clone row (one 16-byte shared load)
 constexpr int kTSide = kRow + 1;     // acceptance table is kTSide x kTSide, indexed 9 n+ + n-
 constexpr int kMaskDeg = 6;          // uniform degrees up to this use mask-indexed thresholds
-constexpr int kWarpsPerYRegion = 8; // one 32-column Y region per 8 warps (pairs not yet met)
+constexpr int kBankRounds = 5;       // a chunk holds at most 32 x this many slots
 constexpr int kMaxClones = 65535;
 constexpr int kMaxPools = 1022;      // pool byte offsets must fit 16 bits
 constexpr int kMaxPoolSize = 255;    // per-pool counts are bytes
@@ -33,23 +34,32 @@ constexpr int64_t kMaxBuckets = 1 << 16;
 // Counter slots of the device statistics block.
 enum Counter {
     kWork = 0, kProgress, kSiteUpdates, kRepsStarted, kRepsRetained, kRepsAborted,
-    kZeroCompletion, kStepLimitHits, kMaxTau, kSumTau, kTauOverAudit, kPackLost, kNumCounters = 16
+    kZeroCompletion, kStepLimitHits, kMaxTau, kSumTau, kTauOverAudit, kNumCounters = 16
 };
 
-// Per-pair statistics record of the one-thread-per-pair kernel, summed into the counters at exit.
+// Per-lane statistics record of the sampling kernel, summed into the counters at exit.
 enum PairStat {
     kPsProgress = 0, kPsStarted, kPsRetained, kPsAborted, kPsZero, kPsLimit, kPsSumTau, kPsMaxTau,
     kPsTauAudit, kPsSiteUpdates, kPairStats = 10
 };
 
-// Per-pair scratch, one contiguous block of 8-byte words per pair: the replication's and the
-// slot's sums G in [0, 2 na) (interleaved per clone in the one-thread-per-pair kernel, in two
-// halves in the lane-group kernel), the statistics record [2 na, 2 na + kPairStats), then the
-// touched-clone bit sets of the replication and of the slot (W 32-bit words each).
+// Lane-group kernel: per-pair scratch, one contiguous block of 8-byte words per pair: the
+// replication's and the slot's sums G in two halves of [0, 2 na), kPairStats words it leaves unused,
+// then the touched-clone bit sets of the replication and of the slot (W 32-bit words each).
 #ifdef __CUDACC__
-__host__ __device__
+#define MCPD_HD __host__ __device__
+#else
+#define MCPD_HD
 #endif
-inline long long pair_words(long long na, long long W) { return 2 * na + kPairStats + W; }
+MCPD_HD inline long long pair_words(long long na, long long W) { return 2 * na + kPairStats + W; }
+// Sampling kernel: an entry is one slot's sums G [na]; a warp's scratch is `bank` entries, the list
+// of those whose pairs are done (two 32-bit words each), and a statistics record per lane.  In 8-byte
+// words.
+MCPD_HD inline long long warp_words(long long bank, long long na) { return bank * na + bank + 32 * kPairStats; }
+#undef MCPD_HD
+
+// Threads per block the sampling kernel is compiled for.
+constexpr int pairs_threads(int deg, bool batch) { return batch || deg == 0 || deg > kMaskDeg ? 640 : 768; }
 
 // Everything the sampler needs, built on the host from (design, y, params).
 struct Tables {
@@ -91,17 +101,16 @@ int build_tables(const mcpd_design *design, const uint8_t *y, const mcpd_params 
 // The run's counters (summed over launches) as mcpd_stats; n_buckets, n_active and kernel_ms are
 // the caller's.
 inline void counters_to_stats(const unsigned long long *c, mcpd_stats *s) {
-    const bool lost = c[kPackLost] != 0;
     s->progress_units = static_cast<int64_t>(c[kProgress]);
-    s->site_updates = lost ? -1 : static_cast<int64_t>(c[kSiteUpdates]);
-    s->reps_started = lost ? -1 : static_cast<int64_t>(c[kRepsStarted]);
-    s->reps_retained = lost ? -1 : static_cast<int64_t>(c[kRepsRetained]);
+    s->site_updates = static_cast<int64_t>(c[kSiteUpdates]);
+    s->reps_started = static_cast<int64_t>(c[kRepsStarted]);
+    s->reps_retained = static_cast<int64_t>(c[kRepsRetained]);
     s->reps_aborted = static_cast<int64_t>(c[kRepsAborted]);
     s->zero_completion_slots = static_cast<int64_t>(c[kZeroCompletion]);
     s->step_limit_hits = static_cast<int64_t>(c[kStepLimitHits]);
     s->max_tau = static_cast<int64_t>(c[kMaxTau]);
     s->sum_tau = static_cast<int64_t>(c[kSumTau]);
-    s->tau_over_audit = lost ? -1 : static_cast<int64_t>(c[kTauOverAudit]);
+    s->tau_over_audit = static_cast<int64_t>(c[kTauOverAudit]);
 }
 
 // The rows and thresholds the single-instance kernel stages (mask-indexed when available).
@@ -119,8 +128,7 @@ struct KParams {
     const uint64_t *Tnu;
     const uint32_t *init_pairs;       // [n_init_pairs]
     int32_t n_init_pairs;
-    long long *pair_scratch;          // [pairs][pair_words(na, W)]
-    uint32_t *y_state;                // [pairs / 32][wpp][32] fallback Y columns (pairs not yet met)
+    long long *pair_scratch;          // [warps][warp_words(bank, na)]
     unsigned long long *S1;           // [nb][na]
     unsigned long long *S2lo;         // [nb][na]
     unsigned long long *S2hi;         // [nb][na]
@@ -140,7 +148,7 @@ struct KParams {
     uint32_t instance;
     int32_t warps;
     uint32_t smem_tables;             // bytes of staged tables at the start of shared memory
-    int32_t y_regions;                // 32-column Y regions in shared memory
+    int32_t bank, chunk;              // entries per warp; slots a warp takes at a time (<= bank)
     uint32_t rk[20];                  // Philox round keys of the seed
     int32_t nT;                       // threshold entries staged (kTSide^2, or mask-indexed)
     int32_t lag;                      // coupled lag L >= 1
@@ -175,6 +183,7 @@ struct InstDesc {
     uint32_t dummy_entry, dummy_word;
     long long P, B, k, ell, L, burn, length, unit, step_limit, slot_offset, tau_audit;
     long long work_begin;             // global index of this instance's first slot in the launch
+    long long unit_begin, units;      // its chunks in the launch: the first one's index, their number
     long long P_total;                // slots in this instance's buckets (the finalize's P)
     unsigned long long seed;
     uint32_t instance;
@@ -186,42 +195,52 @@ struct BParams {
     const InstDesc *insts;
     int32_t n_inst, coupled, scan, max_wpp;
     int32_t lanes, max_m;             // lanes per pair (1, 8, 16, 32); largest pool count
-    long long total_work;
-    long long *pair_scratch;          // [pairs][pair_words(max_na, max_W)]
-    uint32_t *y_state;                // [pairs / 32][max_wpp][32] fallback Y columns
+    long long total_work, total_units;   // slots; chunks
+    long long *pair_scratch;          // [warps][warp_words(bank, max_na)], or per pair pair_words (lane groups)
     unsigned long long *counters;
     int *error;
     int32_t max_na, max_W;
-    int32_t y_regions;                // 32-column Y regions in shared memory
-    int32_t wide;                     // launch the 20-warp variant of the batch kernel
+    int32_t bank;                     // entries per warp (the slots of a chunk, at most)
     int32_t ext;                      // some instance has a meeting cap or a lag > 1
     int32_t udeg;                     // every instance of the class has this uniform degree (0: mixed)
-    int32_t any_init;                 // some instance of the class has a random start
 };
 
-// Launch shape of the one-thread-per-pair kernel (mcpd_kernels.cu).
+// Launch shape of the sampling kernel (mcpd_kernels.cu).
 struct PairsShape {
     int warps = 0;                    // warps per block
-    int y_regions = 0;                // 32-column Y regions per block
-    bool wide = false;                // (batches) the 20-warp variant of the kernel
     int per_sm = 1;                   // resident blocks per SM
     size_t smem = 0;                  // dynamic shared memory per block
 };
-int pairs_y_regions(int coupled, int warps);
-size_t pairs_smem_bytes(size_t tables, int wpp, int warps, int y_regions);
+inline size_t pairs_smem_bytes(size_t tables, int wpp, int warps) {
+    return (tables + static_cast<size_t>(warps) * static_cast<size_t>(wpp) * 128 + 15) / 16 * 16;
+}
+// How `slots` slots are run on `blocks` resident blocks of at most `most` warps: warps per block and
+// slots a warp takes at a time (a chunk).  Slots run for about the same time, so
+//  - more than one round of 32 a warp: the fewest warps that need no more rounds than `most` would,
+//    and chunks of up to kBankRounds rounds (a chunk's pairs fill a warp better, the more slots it has);
+//  - one round: 32 a warp while that keeps kSpreadWarps warps per block busy; below it that many warps
+//    with fewer slots each (a step is shorter, the fewer lanes' branches it carries).
+constexpr int kSpreadWarps = 12;
+struct ChunkShape { int warps, chunk; };
+inline ChunkShape chunk_shape(long long slots, long long blocks, int most, long long bank) {
+    auto up = [](long long a, long long b) { return (a + b - 1) / b; };
+    const long long rounds = up(slots, blocks * most * 32);
+    const long long fills = up(rounds, std::max<long long>(1, bank / 32)), per = up(rounds, fills);
+    long long w = up(slots, fills * per * blocks * 32);
+    w = std::min<long long>(most, std::max<long long>(w, std::min<long long>(kSpreadWarps, up(slots, blocks))));
+    const long long share = up(slots, blocks * w);
+    return {static_cast<int>(w), static_cast<int>(std::min<long long>(bank, up(share, up(share, bank))))};
+}
 // tables: bytes staged at the start of shared memory (0 for batches); wpp: words per column;
-// P: slots of a single instance (0 = do not shape by rounds); warps: requested warps (0 = auto);
-// ext: the run launches the kernel variant with meeting caps and lags > 1; rnd: a single
-// instance with random starts (batches ignore it).
+// P: slots of a single instance (0 = do not shape by rounds); warps: requested warps (0 = auto).
 int pairs_shape(int coupled, int scan, int udeg, bool batch, size_t tables, int wpp, size_t smem_optin,
                 long long P, int sm_count, int warps, bool ext, bool rnd, PairsShape *out);
 
 // The batched sampling-kernel variants (mcpd_batch.cu): the kernel for a class, and the
 // compile-time degree a class of uniform degree udeg runs with (0: the generic build).
 using PairsKernelFn = void (*)(const KParams, const BParams);
-PairsKernelFn pick_batch(int coupled, int scan, int udeg, bool wide, bool ext);
-PairsKernelFn pick_batch_degree(int udeg, bool wide);       // coupled, degrees 4, 5, 7, 8 (mcpd_batch_deg.cu)
-PairsKernelFn pick_batch_ext_degree(int udeg, bool wide);   // coupled, cap / lag, degrees 3..8 (mcpd_batch_ext.cu)
+PairsKernelFn pick_batch(int coupled, int scan, int udeg);
+PairsKernelFn pick_batch_degree(int udeg);                  // coupled, degrees 4, 5, 7, 8 (mcpd_batch_deg.cu)
 int batch_kernel_degree(int coupled, int ext, int udeg);
 
 // Launchers (mcpd_kernels.cu).
@@ -230,8 +249,6 @@ int launch_group(const BParams &bp, int grid, int block, size_t smem, void *stre
 int set_group_smem(int lanes, size_t bytes);
 int group_max_threads(int lanes);
 int group_occupancy(int lanes, int block, size_t smem, int *blocks_per_sm);
-int pairs_max_threads(int coupled, int scan, int udeg, bool batch, bool wide = false, bool ext = false,
-                      bool rnd = true);
 int launch_finalize_batch(const InstDesc *insts, int n_inst, const int32_t *clone_inst,
                           const int32_t *clone_local, long long total_clones, double *est,
                           double *se, void *stream);

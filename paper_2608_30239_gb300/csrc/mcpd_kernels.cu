@@ -1,11 +1,11 @@
 // CUDA kernels (sm_103a) for coupled score-weighted Markov chain pool decoding.
 //
-// pairs_kernel: persistent; one block per SM (or several when the pair state is small); every
-// thread owns one logical slot at a time and runs its coupled pairs (Algorithm 3) back to back
-// under the fixed horizon B with slot refill (Algorithm 4).  Per pair, shared memory holds the
-// two chains' clone bit sets and the per-pool positive counts of both chains (one byte each), laid
-// out word-interleaved over the warp's 32 lanes so that the per-step loads of different pairs never
-// share a bank.  The clone->pool rows, the alias table of the scan weights and the acceptance
+// pairs_kernel (mcpd_pairs.cuh): persistent; one block per SM (or several when the state is small); every
+// warp takes chunks of slots and runs each slot's coupled pairs (Algorithm 3) to their meetings, two
+// lanes to a pair, and then its single chains, a lane each, under the fixed horizon B with slot
+// refill (Algorithm 4).  Per lane, shared memory holds one chain's clone bit set and its
+// per-pool positive counts (one byte each), laid out word-interleaved over the warp's 32 lanes so
+// that the per-step loads of different lanes never share a bank.  The clone->pool rows, the alias table of the scan weights and the acceptance
 // thresholds are staged once per block.  The hot loop is integer-only: a Philox4x32-10 block
 // feeds two steps, the site comes from the alias table, the full conditional from a table lookup
 // indexed by (n+, n-), and the update from a 64-bit integer comparison.  The estimator
@@ -75,30 +75,8 @@ __global__ void philox_kernel(const uint32_t *ctr, uint32_t k0, uint32_t k1, uin
 
 using PairsFn = PairsKernelFn;
 
-PairsFn pick(int coupled, int scan, bool batch, int udeg = 0, bool wide = false, bool ext = false, bool rnd = true) {
-    if (batch) return pick_batch(coupled, scan, batch_kernel_degree(coupled, ext, udeg), wide, ext);
-    if (coupled && !ext && !rnd) {   // the default all-negative start: no random-start check in the loop
-        switch (udeg) {
-            case 3: return pairs_kernel<true, false, false, 3, false, false, false, false>;
-            case 4: return pairs_kernel<true, false, false, 4, false, false, false, false>;
-            case 5: return pairs_kernel<true, false, false, 5, false, false, false, false>;
-            case 6: return pairs_kernel<true, false, false, 6, false, false, false, false>;
-            case 7: return pairs_kernel<true, false, false, 7, false, false, false, false>;
-            case 8: return pairs_kernel<true, false, false, 8, false, false, false, false>;
-            default: return pairs_kernel<true, false, false, 0, false, false, false, false>;
-        }
-    }
-    if (coupled && ext) {
-        switch (udeg) {
-            case 3: return pairs_kernel<true, false, false, 3, false, true>;
-            case 4: return pairs_kernel<true, false, false, 4, false, true>;
-            case 5: return pairs_kernel<true, false, false, 5, false, true>;
-            case 6: return pairs_kernel<true, false, false, 6, false, true>;
-            case 7: return pairs_kernel<true, false, false, 7, false, true>;
-            case 8: return pairs_kernel<true, false, false, 8, false, true>;
-            default: return pairs_kernel<true, false, false, 0, false, true>;
-        }
-    }
+PairsFn pick(int coupled, int scan, bool batch, int udeg) {
+    if (batch) return pick_batch(coupled, scan, batch_kernel_degree(coupled, 0, udeg));
     if (coupled) {
         switch (udeg) {
             case 3: return pairs_kernel<true, false, false, 3>;
@@ -135,16 +113,18 @@ int set_smem(size_t bytes, bool batch) {
             for (int ud = 0; ud <= 8; ++ud) {
                 if (ud && (ud < 3 || (!c && ud > kMaskDeg))) continue;
                 if (batch && ud != batch_kernel_degree(c, 0, ud)) continue;
-                for (int wide = 0; wide <= (batch ? 1 : 0); ++wide)
-                    for (int ext = 0; ext <= c; ++ext)
-                        for (int rnd = 0; rnd <= 1; ++rnd)
-                            if (cudaFuncSetAttribute(pick(c, sc, batch, ud, wide != 0, ext != 0, rnd != 0),
-                                                     cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                     static_cast<int>(bytes)) != cudaSuccess)
-                                return MCPD_ECUDA;
+                if (cudaFuncSetAttribute(pick(c, sc, batch, ud), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         static_cast<int>(bytes)) != cudaSuccess)
+                    return MCPD_ECUDA;
             }
         }
     return batch ? MCPD_OK : set_trace_smem(bytes);
+}
+
+int max_warps(int coupled, int scan, int udeg, bool batch) {
+    cudaFuncAttributes a{};
+    if (cudaFuncGetAttributes(&a, pick(coupled, scan, batch, udeg)) != cudaSuccess) return 16;
+    return a.maxThreadsPerBlock / 32;
 }
 
 }  // namespace
@@ -160,15 +140,13 @@ int pairs_max_smem(int device, size_t *bytes) {
 int launch_pairs(const KParams &kp, int grid, int block, size_t smem, void *stream) {
     if (kp.trace_rec) return launch_pairs_trace(kp, grid, block, smem, stream);
     const BParams none{};
-    const bool ext = kp.capped != 0 || kp.lag > 1;
-    pick(kp.coupled, kp.scan, false, kp.udeg, false, ext, kp.Tnu != nullptr)<<<grid, block, smem,
-                                                                           static_cast<cudaStream_t>(stream)>>>(kp, none);
+    pick(kp.coupled, kp.scan, false, kp.udeg)<<<grid, block, smem, static_cast<cudaStream_t>(stream)>>>(kp, none);
     return cudaGetLastError() == cudaSuccess ? MCPD_OK : MCPD_ECUDA;
 }
 
 int launch_batch(const BParams &bp, int grid, int block, size_t smem, void *stream) {
     const KParams none{};
-    pick(bp.coupled, bp.scan, true, bp.udeg, bp.wide != 0, bp.ext != 0)<<<grid, block, smem, static_cast<cudaStream_t>(stream)>>>(none, bp);
+    pick(bp.coupled, bp.scan, true, bp.udeg)<<<grid, block, smem, static_cast<cudaStream_t>(stream)>>>(none, bp);
     return cudaGetLastError() == cudaSuccess ? MCPD_OK : MCPD_ECUDA;
 }
 
@@ -195,25 +173,10 @@ int launch_philox(const uint32_t *ctr, uint32_t k0, uint32_t k1, uint32_t *out, 
     return cudaGetLastError() == cudaSuccess ? MCPD_OK : MCPD_ECUDA;
 }
 
-int pairs_y_regions(int coupled, int warps) {
-    return coupled ? (warps + kWarpsPerYRegion - 1) / kWarpsPerYRegion : 0;
-}
-
-size_t pairs_smem_bytes(size_t tables, int wpp, int warps, int y_regions) {
-    const size_t b = tables + static_cast<size_t>(warps + y_regions) * static_cast<size_t>(wpp) * 128 +
-                     static_cast<size_t>(y_regions) * 4;
-    return (b + 15) / 16 * 16;
-}
-
 int pairs_shape(int coupled, int scan, int udeg, bool batch, size_t tables, int wpp, size_t smem_optin,
-                long long P, int sm_count, int warps, bool ext, bool rnd, PairsShape *out) {
-    // Batches: the wide variant when the pair state leaves room for more warps than the narrow one
-    // is compiled for.  The thread cap and the occupancy query use the variant the run launches
-    // (ext: the one with meeting caps and lags > 1; rnd: the one that draws random starts).
-    ext = ext && coupled;
-    bool wide = batch;
-    int cap = pairs_max_threads(coupled, scan, udeg, batch, wide, ext, rnd) / 32;
-    auto bytes = [&](int w) { return pairs_smem_bytes(tables, wpp, w, pairs_y_regions(coupled, w)); };
+                long long P, int sm_count, int warps, bool, bool, PairsShape *out) {
+    const int cap = max_warps(coupled, scan, udeg, batch);
+    auto bytes = [&](int w) { return pairs_smem_bytes(tables, wpp, w); };
     auto most = [&](size_t budget) {
         int best = 0;
         for (int w = 1; w <= cap && bytes(w) <= budget; ++w) best = w;
@@ -221,16 +184,12 @@ int pairs_shape(int coupled, int scan, int udeg, bool batch, size_t tables, int 
     };
     auto resident = [&](int w, int *per_sm) {
         *per_sm = 1;
-        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, pick(coupled, scan, batch, udeg, wide, ext, rnd),
-                                                             w * 32, bytes(w)) == cudaSuccess;
+        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, pick(coupled, scan, batch, udeg), w * 32,
+                                                             bytes(w)) == cudaSuccess;
     };
+    // The limit of the interface: the tables and, coupled, both chains of one warp's pairs.
+    if (bytes(coupled ? 2 : 1) > smem_optin) return MCPD_ETOO_LARGE;
     int w1 = most(smem_optin);
-    if (w1 < 1) return MCPD_ETOO_LARGE;
-    if (batch) {
-        const int narrow = pairs_max_threads(coupled, scan, udeg, true, false, ext) / 32;
-        const int target = warps > 0 ? std::min(warps, w1) : w1;
-        if (target <= narrow) { wide = false; cap = narrow; w1 = most(smem_optin); }
-    }
     // The attribute is a permission shared by every launch of the kernel (the classes of a batch
     // have different sizes): allow the device's opt-in maximum.
     if (set_smem(smem_optin, batch) != MCPD_OK) return MCPD_ECUDA;
@@ -247,31 +206,13 @@ int pairs_shape(int coupled, int scan, int udeg, bool batch, size_t tables, int 
             const int w2 = most(smem_optin / 2);
             int per2 = 1;
             if (w2 >= 1 && resident(w2, &per2) && per2 * w2 > s.per_sm * s.warps) { s.warps = w2; s.per_sm = per2; }
-            // Whole rounds of slots: slots run for about the same time, so the fewest warps that
-            // need no more rounds per thread than the widest shape finish at the same time with
-            // no partly filled last round.
-            if (P > 0) {
-                const long long blocks = static_cast<long long>(sm_count) * s.per_sm;
-                const long long rounds = (P + blocks * s.warps * 32 - 1) / (blocks * s.warps * 32);
-                const long long w = (P + rounds * blocks * 32 - 1) / (rounds * blocks * 32);
-                if (w >= 1 && w < s.warps) s.warps = static_cast<int>(w);
-            }
+            if (P > 0) s.warps = chunk_shape(P, static_cast<long long>(sm_count) * s.per_sm, s.warps, 32 * kBankRounds).warps;
         }
     }
-    s.y_regions = pairs_y_regions(coupled, s.warps);
-    s.wide = wide;
     s.smem = bytes(s.warps);
     if (s.per_sm < 1) s.per_sm = 1;
     *out = s;
     return MCPD_OK;
 }
-
-int pairs_max_threads(int coupled, int scan, int udeg, bool batch, bool wide, bool ext, bool rnd) {
-    cudaFuncAttributes a{};
-    if (cudaFuncGetAttributes(&a, pick(coupled, scan, batch, udeg, wide, ext && coupled, rnd)) != cudaSuccess)
-        return 512;
-    return a.maxThreadsPerBlock;
-}
-
 
 }  // namespace mcpd

@@ -116,21 +116,25 @@ extern "C" int mcpd_decode_noalloc(mcpd_ctx *ctx, const mcpd_design *design, con
                                 ctx->sm_count, 0, t.capped || t.lag > 1, !t.Tnu.empty(), &shape);
     if (src == MCPD_ETOO_LARGE) return fail(ctx, src, "instance too large for the one-thread-per-pair layout");
     if (src != MCPD_OK) return fail(ctx, MCPD_ECUDA, "launch shape (cudaFuncSetAttribute / occupancy)");
-    // scratch block (sums, statistics, touched sets) and Y column
-    const size_t per_pair = static_cast<size_t>(pair_words(t.na, t.W)) * 8 + static_cast<size_t>(t.wpp) * 4;
-    // room for the pair scratch and the Y columns, each rounded up to 256 bytes
+    // The limit of this entry point: room for 32 pairs' accumulators of pair_words and a column each.
     if (fixed + 2 * 256 > kNoAllocScratchBytes)
         return fail(ctx, MCPD_ETOO_LARGE, "tables and N*_p buckets exceed the 64 MiB no-alloc scratch");
-    const size_t fit_warps = (kNoAllocScratchBytes - fixed - 2 * 256) / (32 * per_pair);
-    if (fit_warps < 1)
+    const size_t room = kNoAllocScratchBytes - fixed - 2 * 256;
+    if (room < 32 * (static_cast<size_t>(pair_words(t.na, t.W)) * 8 + static_cast<size_t>(t.wpp) * 4))
         return fail(ctx, MCPD_ETOO_LARGE, "not even one warp of pair accumulators fits the 64 MiB no-alloc scratch");
-    const int warps = static_cast<int>(std::min<size_t>(shape.warps, fit_warps));
-    const int y_regions = pairs_y_regions(t.coupled, warps);
-    const size_t smem = pairs_smem_bytes(tables, t.wpp, warps, y_regions);
-    const int grid = static_cast<int>(std::min<size_t>(static_cast<size_t>(ctx->sm_count) * shape.per_sm, fit_warps / warps));
-    const size_t pairs = static_cast<size_t>(grid) * warps * 32;
-    const size_t o_pair = take(pairs * static_cast<size_t>(pair_words(t.na, t.W)) * 8);
-    const size_t o_y = take(pairs * t.wpp * 4);
+    // Chunks in fours, and only the warps they fill (every call clears the scratch it uses); then fewer
+    // warps, and fewer blocks, with larger chunks until their banks fit.
+    int warps = shape.warps, grid = ctx->sm_count * shape.per_sm, chunk = 1;
+    auto up = [](long long a, long long b) { return (a + b - 1) / b; };
+    for (bool first = true;; first = false) {
+        chunk = static_cast<int>(std::min<long long>(32, 4 * up(t.P, 4ll * grid * warps)));
+        if (first) warps = static_cast<int>(std::min<long long>(warps, up(t.P, static_cast<long long>(grid) * chunk)));
+        if (static_cast<size_t>(grid) * warps * warp_words(chunk, t.na) * 8 <= room || (grid == 1 && warps == 1)) break;
+        if (warps > 1) --warps; else --grid;
+    }
+    const size_t smem = pairs_smem_bytes(tables, t.wpp, warps);
+    const size_t all_warps = static_cast<size_t>(grid) * warps;
+    const size_t o_pair = take(all_warps * static_cast<size_t>(warp_words(chunk, t.na)) * 8);
     if (off > kNoAllocScratchBytes) return fail(ctx, MCPD_ETOO_LARGE, "no-alloc scratch layout overflow");
 
     unsigned char *b = static_cast<unsigned char *>(base);
@@ -151,7 +155,6 @@ extern "C" int mcpd_decode_noalloc(mcpd_ctx *ctx, const mcpd_design *design, con
     kp.init_pairs = reinterpret_cast<const uint32_t *>(b + o_init);
     kp.n_init_pairs = static_cast<int32_t>(t.init_pairs.size());
     kp.pair_scratch = reinterpret_cast<long long *>(b + o_pair);
-    kp.y_state = reinterpret_cast<uint32_t *>(b + o_y);
     kp.S1 = reinterpret_cast<unsigned long long *>(b + o_S1);
     kp.S2lo = reinterpret_cast<unsigned long long *>(b + o_S2lo);
     kp.S2hi = reinterpret_cast<unsigned long long *>(b + o_S2hi);
@@ -170,7 +173,8 @@ extern "C" int mcpd_decode_noalloc(mcpd_ctx *ctx, const mcpd_design *design, con
     kp.seed = t.seed; philox_round_keys(t.seed, kp.rk); kp.instance = t.instance; kp.warps = warps;
     kp.smem_tables = static_cast<uint32_t>(tables);
     kp.nT = static_cast<int32_t>(kernel_T(t).size());
-    kp.y_regions = y_regions;
+    kp.bank = chunk;
+    kp.chunk = chunk;
     if (launch_pairs(kp, grid, warps * 32, smem, s) != MCPD_OK)
         return fail(ctx, MCPD_ECUDA, std::string("pairs kernel launch: ") + cudaGetErrorString(cudaGetLastError()));
     if (launch_finalize(kp.S1, kp.S2lo, kp.S2hi, t.na, static_cast<int>(t.nb), t.P, t.L, est_dev, se_dev, s) != MCPD_OK)
@@ -185,7 +189,7 @@ extern "C" int mcpd_decode_noalloc(mcpd_ctx *ctx, const mcpd_design *design, con
         counters_to_stats(c, stats);
         stats->n_buckets = t.nb;
         stats->n_active = t.na;
-        stats->resident_pairs = static_cast<int64_t>(pairs);
+        stats->resident_pairs = static_cast<int64_t>(all_warps) * std::min(32, chunk);
     }
     if (error) return fail(ctx, MCPD_ESTEP_LIMIT, "a pair reached the step limit without meeting");
     return MCPD_OK;

@@ -12,44 +12,33 @@ namespace {
 
 using TraceFn = void (*)(const KParams, const BParams);
 
-TraceFn pick_trace(int coupled, int scan, int udeg, bool ext) {
+TraceFn pick_trace(int coupled, int scan, int udeg) {
     if (!coupled && scan == MCPD_SCAN_SYSTEMATIC) {
         switch (udeg) {
-            case 3: return pairs_kernel<false, true, false, 3, false, false, true>;
-            case 4: return pairs_kernel<false, true, false, 4, false, false, true>;
-            case 5: return pairs_kernel<false, true, false, 5, false, false, true>;
-            case 6: return pairs_kernel<false, true, false, 6, false, false, true>;
-            default: return pairs_kernel<false, true, false, 0, false, false, true>;
+            case 3: return pairs_kernel<false, true, false, 3, true>;
+            case 4: return pairs_kernel<false, true, false, 4, true>;
+            case 5: return pairs_kernel<false, true, false, 5, true>;
+            case 6: return pairs_kernel<false, true, false, 6, true>;
+            default: return pairs_kernel<false, true, false, 0, true>;
         }
     }
     if (!coupled) {
         switch (udeg) {
-            case 3: return pairs_kernel<false, false, false, 3, false, false, true>;
-            case 4: return pairs_kernel<false, false, false, 4, false, false, true>;
-            case 5: return pairs_kernel<false, false, false, 5, false, false, true>;
-            case 6: return pairs_kernel<false, false, false, 6, false, false, true>;
-            default: return pairs_kernel<false, false, false, 0, false, false, true>;
-        }
-    }
-    if (ext) {
-        switch (udeg) {
-            case 3: return pairs_kernel<true, false, false, 3, false, true, true>;
-            case 4: return pairs_kernel<true, false, false, 4, false, true, true>;
-            case 5: return pairs_kernel<true, false, false, 5, false, true, true>;
-            case 6: return pairs_kernel<true, false, false, 6, false, true, true>;
-            case 7: return pairs_kernel<true, false, false, 7, false, true, true>;
-            case 8: return pairs_kernel<true, false, false, 8, false, true, true>;
-            default: return pairs_kernel<true, false, false, 0, false, true, true>;
+            case 3: return pairs_kernel<false, false, false, 3, true>;
+            case 4: return pairs_kernel<false, false, false, 4, true>;
+            case 5: return pairs_kernel<false, false, false, 5, true>;
+            case 6: return pairs_kernel<false, false, false, 6, true>;
+            default: return pairs_kernel<false, false, false, 0, true>;
         }
     }
     switch (udeg) {
-        case 3: return pairs_kernel<true, false, false, 3, false, false, true>;
-        case 4: return pairs_kernel<true, false, false, 4, false, false, true>;
-        case 5: return pairs_kernel<true, false, false, 5, false, false, true>;
-        case 6: return pairs_kernel<true, false, false, 6, false, false, true>;
-        case 7: return pairs_kernel<true, false, false, 7, false, false, true>;
-        case 8: return pairs_kernel<true, false, false, 8, false, false, true>;
-        default: return pairs_kernel<true, false, false, 0, false, false, true>;
+        case 3: return pairs_kernel<true, false, false, 3, true>;
+        case 4: return pairs_kernel<true, false, false, 4, true>;
+        case 5: return pairs_kernel<true, false, false, 5, true>;
+        case 6: return pairs_kernel<true, false, false, 6, true>;
+        case 7: return pairs_kernel<true, false, false, 7, true>;
+        case 8: return pairs_kernel<true, false, false, 8, true>;
+        default: return pairs_kernel<true, false, false, 0, true>;
     }
 }
 
@@ -59,13 +48,12 @@ int set_trace_smem(size_t bytes) {
     for (int c = 0; c <= 1; ++c)
         for (int sc : {MCPD_SCAN_SCORE, MCPD_SCAN_SYSTEMATIC}) {
             if (c && sc == MCPD_SCAN_SYSTEMATIC) continue;
-            for (int ext = 0; ext <= c; ++ext)
-                for (int ud = 0; ud <= 8; ++ud) {
-                    if (ud == 1 || ud == 2 || (!c && ud > kMaskDeg)) continue;
-                    if (cudaFuncSetAttribute(pick_trace(c, sc, ud, ext != 0), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             static_cast<int>(bytes)) != cudaSuccess)
-                        return MCPD_ECUDA;
-                }
+            for (int ud = 0; ud <= 8; ++ud) {
+                if (ud == 1 || ud == 2 || (!c && ud > kMaskDeg)) continue;
+                if (cudaFuncSetAttribute(pick_trace(c, sc, ud), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         static_cast<int>(bytes)) != cudaSuccess)
+                    return MCPD_ECUDA;
+            }
         }
     return MCPD_OK;
 }
@@ -73,8 +61,7 @@ int set_trace_smem(size_t bytes) {
 int launch_pairs_trace(const KParams &kp, int grid, int block, size_t smem, void *stream) {
     if (!kp.trace_rec || kp.trace_stride <= 0) return MCPD_EINVAL;
     const BParams none{};
-    const bool ext = kp.coupled && (kp.capped != 0 || kp.lag > 1);
-    pick_trace(kp.coupled, kp.scan, kp.udeg, ext)<<<grid, block, smem, static_cast<cudaStream_t>(stream)>>>(kp, none);
+    pick_trace(kp.coupled, kp.scan, kp.udeg)<<<grid, block, smem, static_cast<cudaStream_t>(stream)>>>(kp, none);
     return cudaGetLastError() == cudaSuccess ? MCPD_OK : MCPD_ECUDA;
 }
 
