@@ -68,7 +68,7 @@ struct Tables {
     bool coupled = true;
     std::vector<int32_t> active;      // [na] original index of active clone a, ascending
     std::vector<uint64_t> alias;      // [na] prob (low 32) | alias index (high 32)
-    std::vector<uint16_t> rows;       // [na * kRow] byte offset of the pool's count | y << 15
+    std::vector<uint16_t> rows;       // [na * kRow] byte offsets of the pools' counts: see build_tables
     std::vector<uint16_t> rows_pool;  // [na * kRow] pool id | y << 15, 0xFFFF past the clone's pools
     std::vector<uint64_t> T;          // [kTSide * kTSide]
     std::vector<uint64_t> Tnu;        // [na] or empty

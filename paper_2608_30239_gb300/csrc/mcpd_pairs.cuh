@@ -121,10 +121,11 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
     MCPD_FIELD(v_bcount, reinterpret_cast<unsigned long long *>(__ldg(reinterpret_cast<const unsigned long long *>(&desc->bcount))), p.bcount);
 #undef MCPD_FIELD
     auto clamp32 = [](long long v) -> uint32_t { return v < 0 ? 0u : (v > 0xFFFFFFFFll ? 0xFFFFFFFFu : static_cast<uint32_t>(v)); };
-    // Uniform degree 3..kMaskDeg (every clone of the instance, or of every instance of a batched
-    // class, sits in exactly DEG pools): rows hold plain offsets with the clone's positive-outcome
-    // pools first and their number in the last entry; thresholds are indexed
-    // npos * 64 + (mask of deciding pools).
+    // Rows list a clone's positive-outcome pools first.  Uniform degree 3..kMaskDeg (every clone of
+    // the instance, or of every instance of a batched class, sits in exactly DEG pools): their number
+    // is the last entry, and thresholds are indexed npos * 64 + (mask of deciding pools).  Other
+    // degrees fill all eight entries: the number sits in bits of entry 0 that an offset leaves
+    // clear, and n+ and n- are counted from the mask.
     constexpr bool MASKT = DEG >= 3 && DEG <= kMaskDeg;
     auto derive = [&]() {
         ws0 = clamp32(COUPLED ? v_k() : v_burn());
@@ -154,7 +155,7 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
         else return reinterpret_cast<const uint32_t *>(sT)[2 * i];
     };
     auto entries = [&](const uint4 &row, uint32_t *ent) {
-        ent[0] = row.x & 0xFFFFu; ent[1] = row.x >> 16; ent[2] = row.y & 0xFFFFu; ent[3] = row.y >> 16;
+        ent[0] = row.x & (MASKT ? 0xFFFFu : 0xFF83u); ent[1] = row.x >> 16; ent[2] = row.y & 0xFFFFu; ent[3] = row.y >> 16;
         ent[4] = row.z & 0xFFFFu; ent[5] = row.z >> 16; ent[6] = row.w & 0xFFFFu; ent[7] = row.w >> 16;
     };
     // Entry l of a row is a real pool (not past the clone's degree, not the padding pool).
@@ -202,12 +203,13 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
         for (int l = 0; l < kRow; ++l) {
             s.c[l] = 0u;
             if (l < NE && (DEG > 0 || l < deg)) {
-                s.c[l] = cbase[MASKT ? s.ent[l] : s.ent[l] & 0x7FFFu];
-                if constexpr (MASKT) { if (s.c[l] == s.z) s.ix |= 1u << l; }
-                else if (s.c[l] == s.z) s.ix += (s.ent[l] >> 15) ? 9u : 1u;
+                s.c[l] = cbase[s.ent[l]];
+                if (s.c[l] == s.z) s.ix |= 1u << l;
             }
         }
-        if constexpr (MASKT) s.ix += s.ent[kRow - 1] << 6;        // row of the positive-pool count
+        // the threshold's index: of the mask in the positive pools' row, or 9 n+ + n-
+        if constexpr (MASKT) s.ix += s.ent[kRow - 1] << 6;
+        else s.ix = __popc(s.ix) + 8u * __popc(s.ix & ~(0xFFFFFFFFu << ((row.x >> 2) & 15u)));
         s.th = tHi(s.ix);
     };
     auto may = [&](const Site &s, uint32_t wu) -> bool { return s.z ? wu >= s.th : wu <= s.th; };
@@ -222,7 +224,7 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
         const uint32_t delta = s.z ? 0xFFu : 1u;
 #pragma unroll
         for (int l = 0; l < kRow; ++l)
-            if (real(l, s.ent)) cbase[MASKT ? s.ent[l] : s.ent[l] & 0x7FFFu] = static_cast<unsigned char>(s.c[l] + delta);
+            if (real(l, s.ent)) cbase[s.ent[l]] = static_cast<unsigned char>(s.c[l] + delta);
     };
     // Random start Z_0 ~ prod Bernoulli(nu_i) of lane src's new replication, drawn by the whole
     // warp: the lanes take the clone pairs that have some nu_i > 0 (one Philox block each, tag 1, counter
@@ -252,7 +254,7 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
 #pragma unroll
                     for (int l = 0; l < kRow; ++l) {
                         if (!real(l, ent)) continue;
-                        const uint32_t off = MASKT ? ent[l] : (ent[l] & 0x7FFFu);
+                        const uint32_t off = ent[l];
                         atomicAdd(reinterpret_cast<uint32_t *>(cb_s + (off & ~3u)), 1u << (8u * (off & 3u)));
                     }
                 }

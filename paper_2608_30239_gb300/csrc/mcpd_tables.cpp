@@ -219,35 +219,39 @@ int build_tables(const mcpd_design *d, const uint8_t *y, const mcpd_params *prm,
     t.dummy_entry = static_cast<uint16_t>(count_offset(m));
     t.dummy_word_index = t.W + (m >> 2);
     t.dummy_word = 2u << (8 * (m & 3));
+    // A row lists the clone's positive-outcome pools first, as count offsets, then the others, then the
+    // padding pool (count 2: it never decides).  The number of positive ones goes into bits 2-5 of
+    // entry 0 (an offset has bits 2-6 clear), so a mask of deciding pools gives (n+, n-).
     t.rows.assign(static_cast<size_t>(na) * kRow, t.dummy_entry);
     t.rows_pool.assign(static_cast<size_t>(na) * kRow, 0xFFFFu);
-    for (int32_t a = 0; a < na; ++a) {
-        int32_t i = t.active[a];
-        int32_t l = 0;
-        for (int32_t e = d->clone_ptr[i]; e < d->clone_ptr[i + 1]; ++e, ++l) {
-            int32_t j = d->clone_pools[e];
-            t.rows[static_cast<size_t>(a) * kRow + l] = static_cast<uint16_t>(count_offset(j) | (y[j] ? 0x8000u : 0u));
-            t.rows_pool[static_cast<size_t>(a) * kRow + l] = static_cast<uint16_t>(j | (y[j] ? 0x8000u : 0u));
-        }
-    }
-    // Runs with a uniform degree 3 <= d <= kMaskDeg (single-instance kernels compiled for d, coupled
-    // or not): each row lists the clone's positive-outcome pools first, as plain count offsets,
-    // with their number in entry kRow - 1; T_mask[npos][m] = T[9 n+ + n-] for the mask m of
-    // deciding pools (n+ of them among the first npos entries, n- among the rest).  The same
-    // thresholds, indexed without per-entry codes.
+    // Uniform degree 3 <= d <= kMaskDeg (kernels compiled for d): plain offsets, the number of
+    // positive pools in entry kRow - 1, and T_mask[npos][m] = T[9 n+ + n-] for the mask m of deciding
+    // pools (n+ of them among the first npos entries, n- among the rest).
     t.rows_mask.clear();
     t.T_mask.clear();
-    if (t.udeg >= 3 && t.udeg <= kMaskDeg) {                  // the kernels compiled for degree d
-        t.rows_mask.assign(static_cast<size_t>(na) * kRow, 0);
-        for (int32_t a = 0; a < na; ++a) {
-            const uint16_t *src = &t.rows[static_cast<size_t>(a) * kRow];
+    const bool masked = t.udeg >= 3 && t.udeg <= kMaskDeg;
+    if (masked) t.rows_mask.assign(static_cast<size_t>(na) * kRow, 0);
+    for (int32_t a = 0; a < na; ++a) {
+        const int32_t i = t.active[a], e0 = d->clone_ptr[i], e1 = d->clone_ptr[i + 1];
+        uint16_t *row = &t.rows[static_cast<size_t>(a) * kRow];
+        int32_t l = 0, npos = 0;
+        for (int32_t pass = 1; pass >= 0; --pass) {
+            for (int32_t e = e0; e < e1; ++e)
+                if (y[d->clone_pools[e]] == pass) row[l++] = static_cast<uint16_t>(count_offset(d->clone_pools[e]));
+            if (pass) npos = l;
+        }
+        for (int32_t e = e0; e < e1; ++e) {
+            const int32_t j = d->clone_pools[e];
+            t.rows_pool[static_cast<size_t>(a) * kRow + (e - e0)] = static_cast<uint16_t>(j | (y[j] ? 0x8000u : 0u));
+        }
+        if (masked) {
             uint16_t *dst = &t.rows_mask[static_cast<size_t>(a) * kRow];
-            int32_t fill = 0;
-            for (int32_t l = 0; l < t.udeg; ++l) if (src[l] & 0x8000u) dst[fill++] = static_cast<uint16_t>(src[l] & 0x7FFFu);
-            const int32_t npos = fill;
-            for (int32_t l = 0; l < t.udeg; ++l) if (!(src[l] & 0x8000u)) dst[fill++] = src[l];
+            std::copy(row, row + t.udeg, dst);
             dst[kRow - 1] = static_cast<uint16_t>(npos);
         }
+        row[0] = static_cast<uint16_t>(row[0] | (npos << 2));
+    }
+    if (masked) {
         t.T_mask.assign(static_cast<size_t>(kMaskDeg + 1) * 64, 0);
         for (int32_t npos = 0; npos <= kMaskDeg; ++npos)
             for (int32_t mask = 0; mask < 64; ++mask) {
