@@ -160,6 +160,48 @@ static int assign_classes(const std::vector<mcpd::Tables> &t, int want_classes, 
     return n_cls_out;
 }
 
+// The launches of a batch: classes that the library chose (`split`) are cut once more by pair state,
+// to four launches per degree group, if one launch per class would not fit the GPU at once.
+// A launch sizes every warp's columns for its largest instance, so few slots in few classes left
+// the small instances' warps with a large one's columns and the blocks in two waves: 128 instances
+// of 200 to 5000 clones, 512 slots each, took 98 ms in 5 launches, 88 ms in 20.  Replaces class by launch in *cls_of and
+// returns each launch's class.  Results do not depend on the launches.
+static std::vector<int32_t> cut_launches(const std::vector<mcpd::Tables> &t, bool split, int n_cls, int sm_count,
+                                         size_t smem, std::vector<int32_t> *cls_of) {
+    const int32_t n_inst = static_cast<int32_t>(t.size());
+    std::vector<std::vector<int32_t>> of(n_cls);
+    for (int32_t i = 0; i < n_inst; ++i) of[(*cls_of)[i]].push_back(i);
+    double columns = 0.0;                       // bytes of all slots' columns, one launch per class
+    std::vector<int> degrees;
+    for (const auto &c : of) {
+        int32_t wpp = 0;
+        double slots = 0.0;
+        for (int32_t i : c) { wpp = std::max(wpp, t[i].wpp); slots += static_cast<double>(t[i].P); }
+        columns += slots * wpp * 4.0;
+        const int d = mcpd::batch_kernel_degree(t[0].coupled ? 1 : 0, 0, t[c[0]].udeg);
+        if (std::find(degrees.begin(), degrees.end(), d) == degrees.end()) degrees.push_back(d);
+    }
+    const bool cut = split && columns > static_cast<double>(sm_count) * smem;
+    const int per = cut ? std::max(1, 4 * static_cast<int>(degrees.size()) / n_cls) : 1;
+    std::vector<int32_t> cls_of_launch;
+    for (int c = 0; c < n_cls; ++c) {
+        auto &m = of[c];
+        std::stable_sort(m.begin(), m.end(), [&](int32_t a, int32_t b) { return t[a].wpp > t[b].wpp; });
+        auto work = [&](int32_t i) { return static_cast<double>(t[i].P) * static_cast<double>(std::max(t[i].B, t[i].unit)); };
+        double total = 0.0, acc = 0.0;
+        for (int32_t i : m) total += work(i);
+        const int parts = std::min<int>(per, static_cast<int>(m.size()));
+        int last = -1;
+        for (int32_t i : m) {
+            const int k = std::min(parts - 1, static_cast<int>(total > 0 ? acc / total * parts : 0.0));
+            if (k != last) { cls_of_launch.push_back(c); last = k; }
+            (*cls_of)[i] = static_cast<int32_t>(cls_of_launch.size()) - 1;
+            acc += work(i);
+        }
+    }
+    return cls_of_launch;
+}
+
 extern "C" {
 
 int mcpd_ctx_create(int device, void *cuda_stream, mcpd_ctx **out) {
@@ -541,8 +583,9 @@ int mcpd_philox_device(mcpd_ctx *ctx, const uint32_t *ctr_dev, uint32_t key0, ui
 // ------------------------------------------------------------------------------------------
 // Batched decoding: many instances of uneven size in one persistent launch.
 
-// One size class of a batch: instances with similar pair state, launched together so that the
-// launch shape (warps per block) fits their columns rather than the largest instance's.
+// One launch of a batch (a class, or a part of one: cut_launches): instances with similar pair state,
+// launched together so that the launch shape (warps per block) fits their columns rather than the
+// largest instance's.
 struct BatchClass {
     int32_t first = 0, count = 0;      // positions [first, first + count) of the launch order
     mcpd::BParams bp{};                // this class's launch arguments (insts = d_insts + first)
@@ -560,7 +603,11 @@ struct mcpd_batch {
     std::vector<int64_t> out_offset;       // [n + 1] offsets of each instance's clones in est/se
     std::vector<int64_t> bucket_offset;    // [n] offsets of each instance's buckets (in nb*na units)
     std::vector<int64_t> count_offset;     // [n]
-    std::vector<BatchClass> cls;
+    std::vector<BatchClass> cls;           // the launches, in launch order
+    std::vector<int32_t> class_of_launch;  // the class each belongs to
+    std::vector<int32_t> enqueue_order;    // longest slots first: their blocks start at once, and the
+                                           // short ones fill the SMs that come free
+    int n_classes = 0;
     int32_t n_inst = 0, lanes = 1;
     bool coupled = true;
     mcpd::InstDesc *d_insts = nullptr;
@@ -731,7 +778,7 @@ int batch_enqueue(mcpd_ctx *ctx, mcpd_batch *b, double *est_dev, double *se_dev,
         }
     }
     CU(cudaEventRecord(b->fork, s));
-    for (size_t k = 0; k < b->cls.size(); ++k) {
+    for (const int32_t k : b->enqueue_order) {
         const BatchClass &c = b->cls[k];
         const cudaStream_t cs = b->cls_streams[k];
         CU(cudaStreamWaitEvent(cs, b->fork, 0));
@@ -798,7 +845,9 @@ int mcpd_batch_create(mcpd_ctx *ctx, int32_t n_inst, const mcpd_design *designs,
     if (cudaSetDevice(ctx->device) != cudaSuccess) { mcpd_batch_destroy(b); return set_err(ctx, MCPD_ECUDA, "cudaSetDevice"); }
 
     std::vector<int32_t> cls_of;
-    int n_cls = assign_classes(b->t, want_classes, ctx->sm_count, &cls_of);
+    b->n_classes = assign_classes(b->t, want_classes, ctx->sm_count, &cls_of);
+    b->class_of_launch = cut_launches(b->t, want_classes == 0, b->n_classes, ctx->sm_count, ctx->smem_optin, &cls_of);
+    const int n_cls = static_cast<int>(b->class_of_launch.size());
     int64_t total_slots = 0;
     for (int32_t i = 0; i < n_inst; ++i) total_slots += b->t[i].P;
     // Launch order: class by class; within a class, 0 = input order, 1 = longest slots first.
@@ -913,6 +962,14 @@ int mcpd_batch_create(mcpd_ctx *ctx, int32_t n_inst, const mcpd_design *designs,
     CU_OR(cudaMemcpyAsync(b->d_insts, b->insts.data(), sizeof(mcpd::InstDesc) * n_inst, cudaMemcpyHostToDevice, ctx->stream), mcpd_batch_destroy(b));
     b->insts0 = b->insts;
     for (const BatchClass &c : b->cls) b->total_work0.push_back(c.bp.total_work);
+    {
+        std::vector<int64_t> longest(n_cls, 0);
+        for (int32_t i = 0; i < n_inst; ++i)
+            longest[cls_of[i]] = std::max(longest[cls_of[i]], std::max(b->t[i].B, b->t[i].unit));
+        for (int c = 0; c < n_cls; ++c) b->enqueue_order.push_back(c);
+        std::stable_sort(b->enqueue_order.begin(), b->enqueue_order.end(),
+                         [&](int32_t a, int32_t c) { return longest[a] > longest[c]; });
+    }
     CU_OR(cudaMemcpyAsync(b->d_clone_inst, ci.data(), ci.size() * 4, cudaMemcpyHostToDevice, ctx->stream), mcpd_batch_destroy(b));
     CU_OR(cudaMemcpyAsync(b->d_clone_local, cl.data(), cl.size() * 4, cudaMemcpyHostToDevice, ctx->stream), mcpd_batch_destroy(b));
     if ((rc = batch_shape(ctx, b, 0)) != MCPD_OK) { mcpd_batch_destroy(b); return rc; }
@@ -935,17 +992,20 @@ int mcpd_batch_info(const mcpd_batch *b, int64_t info[16]) {
     std::memset(info, 0, 16 * sizeof(int64_t));
     int32_t max_na = 0;
     int64_t pairs = 0, wmax = 0, ext = 0, degree_builds = 0;
-    for (const BatchClass &c : b->cls) {
+    std::vector<char> is_ext(b->n_classes, 0), degree(b->n_classes, b->lanes == 1);
+    for (size_t k = 0; k < b->cls.size(); ++k) {
+        const BatchClass &c = b->cls[k];
         max_na = std::max(max_na, c.bp.max_na);
         pairs = std::max<int64_t>(pairs, c.pairs);
         wmax = std::max<int64_t>(wmax, c.warps);
-        ext += c.bp.ext;
-        if (b->lanes == 1 && mcpd::batch_kernel_degree(c.bp.coupled, c.bp.ext, c.bp.udeg) > 0) ++degree_builds;
+        if (c.bp.ext) is_ext[b->class_of_launch[k]] = 1;
+        if (mcpd::batch_kernel_degree(c.bp.coupled, c.bp.ext, c.bp.udeg) == 0) degree[b->class_of_launch[k]] = 0;
     }
+    for (int k = 0; k < b->n_classes; ++k) { ext += is_ext[k]; degree_builds += degree[k]; }
     const BatchClass &c0 = b->cls[0];
     info[0] = b->total_active; info[1] = b->n_inst; info[2] = b->total_slots; info[3] = max_na;
     info[4] = c0.warps; info[5] = c0.grid; info[6] = pairs; info[7] = static_cast<int64_t>(c0.smem);
-    info[8] = b->lanes; info[9] = static_cast<int64_t>(b->cls.size()); info[10] = wmax; info[11] = ext;
+    info[8] = b->lanes; info[9] = b->n_classes; info[10] = wmax; info[11] = ext;
     info[12] = degree_builds;
     return MCPD_OK;
 }
