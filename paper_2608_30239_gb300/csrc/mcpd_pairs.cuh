@@ -175,17 +175,32 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
     int32_t *trec = nullptr;              // TRACE: the record of the current replication
     uint32_t trace_from = 0;              // TRACE: the single run records from its pair's meeting on
 
-    // The site a step word selects (alias draw).
-    auto site_of = [&](uint32_t ws) -> uint32_t {
-        const unsigned long long prod = static_cast<unsigned long long>(ws) * static_cast<uint32_t>(na);
-        const uint32_t col = static_cast<uint32_t>(prod >> 32), coin = static_cast<uint32_t>(prod);
-        const unsigned long long e = aliasAt(col);
-        return coin < static_cast<uint32_t>(e) ? col : static_cast<uint32_t>(e >> 32);
-    };
-    // The site of the current step and its row, drawn ahead: they depend on the step words only,
-    // so the next step's alias and row loads overlap this step's work.
-    uint32_t I_cur = 0;
+    // The site a step word selects (alias draw), and its row, ahead of the step: they depend on the
+    // step words only.  Tables in shared memory: one step ahead.  A batch's tables come from L2 (some
+    // 300 cycles a load), and the row's address waits for the alias word: the alias word two steps
+    // ahead, the row one.
+    uint32_t I_cur = 0, col_next = 0, coin_next = 0;
     uint4 row_cur = make_uint4(0u, 0u, 0u, 0u);
+    unsigned long long e_next = 0;
+    auto column = [&](uint32_t ws) {
+        const unsigned long long prod = static_cast<unsigned long long>(ws) * static_cast<uint32_t>(na);
+        col_next = static_cast<uint32_t>(prod >> 32);
+        coin_next = static_cast<uint32_t>(prod);
+        e_next = aliasAt(col_next);
+    };
+    auto site = [&]() {
+        I_cur = coin_next < static_cast<uint32_t>(e_next) ? col_next : static_cast<uint32_t>(e_next >> 32);
+        row_cur = rowAt(I_cur);
+    };
+    auto ahead = [&](uint32_t ws) {       // ws: the site word of the next step, in a batch of the one after
+        if constexpr (BATCH) { site(); column(ws); }
+        else { column(ws); site(); }
+    };
+    auto first_site = [&](const uint4 &blk) {
+        column(blk.x);
+        site();
+        if constexpr (BATCH) column(blk.z);
+    };
 
     // One step of one chain: the site's bit z and the counts c of its pools in the lane's column; a
     // pool decides when it holds no other positive (c - z = 0); the threshold the deciding pools
@@ -417,7 +432,7 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
             const uint32_t lag = v_lag();
             const bool quick = ell <= v_step_limit();   // (else a pair that has met runs into its limit)
             uint32_t taken = 0;           // slots handed to pairs
-            uint4 blk = make_uint4(0u, 0u, 0u, 0u);
+            uint4 blk = make_uint4(0u, 0u, 0u, 0u), nxt = blk;
             auto draw = [&](uint32_t c0) -> uint4 {
                 if constexpr (BATCH) return philox10(make_uint4(c0, r, slot_g, instance), k0, k1);
                 else return philox10_rk(make_uint4(c0, r, slot_g, instance), p.rk);
@@ -428,8 +443,7 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
                 Site s;
                 s.I = I_cur;
                 const uint4 row = row_cur;
-                I_cur = site_of(ws_next);
-                row_cur = rowAt(I_cur);
+                ahead(ws_next);
                 look(s, row);
                 bool f = on && t >= still && may(s, wu);
                 if (TRACE || __any_sync(FULL, f)) {
@@ -623,16 +637,24 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
                         trace_at();
                         on = true;
                         blk = draw(0);
-                        I_cur = site_of(blk.x);
-                        row_cur = rowAt(I_cur);
+                        if constexpr (BATCH) nxt = draw(1);
+                        first_site(blk);
                     }
                     if (!__any_sync(FULL, on)) break;
                 }
                 was_on = on;
-                const uint4 nxt = draw((t >> 1) + 1);
-                step(blk.z, blk.y);
-                step(nxt.x, blk.w);
-                blk = nxt;
+                if constexpr (BATCH) {
+                    const uint4 after = draw((t >> 1) + 2);
+                    step(nxt.x, blk.y);
+                    step(nxt.z, blk.w);
+                    blk = nxt;
+                    nxt = after;
+                } else {
+                    nxt = draw((t >> 1) + 1);
+                    step(blk.z, blk.y);
+                    step(nxt.x, blk.w);
+                    blk = nxt;
+                }
             }
         } else {
             ready = cnt;
@@ -695,8 +717,7 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
                     } else {
                         s.I = I_cur;
                         row = row_cur;
-                        I_cur = site_of(ws_next);
-                        row_cur = rowAt(I_cur);
+                        ahead(ws_next);
                     }
                     look(s, row);
                     const bool m = may(s, wu);
@@ -711,14 +732,25 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
                     }
                 };
                 uint4 blk = draw(0);
-                if (!SYSTEMATIC) { I_cur = site_of(blk.x); row_cur = rowAt(I_cur); }
+                if (!SYSTEMATIC) first_site(blk);
                 uint32_t time = 0;
-                for (; time + 2 <= ell; time += 2) {
-                    // both steps of the block inlined, the next block drawn between them
-                    step(blk.z, blk.y, time);
-                    const uint4 nxt = draw((time >> 1) + 1);
-                    step(nxt.x, blk.w, time + 1);
-                    blk = nxt;
+                // both steps of a block inlined, the next block drawn between them
+                if constexpr (BATCH) {
+                    uint4 nxt = draw(1);
+                    for (; time + 2 <= ell; time += 2) {
+                        step(nxt.x, blk.y, time);
+                        const uint4 after = draw((time >> 1) + 2);
+                        step(nxt.z, blk.w, time + 1);
+                        blk = nxt;
+                        nxt = after;
+                    }
+                } else {
+                    for (; time + 2 <= ell; time += 2) {
+                        step(blk.z, blk.y, time);
+                        const uint4 nxt = draw((time >> 1) + 1);
+                        step(nxt.x, blk.w, time + 1);
+                        blk = nxt;
+                    }
                 }
                 if (ell & 1u) step(blk.z, blk.y, time);
                 // The closing terms w(l) of X_l's bits, and the column back to empty: every lane its
