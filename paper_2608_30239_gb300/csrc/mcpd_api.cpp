@@ -279,7 +279,7 @@ int mcpd_plan_create(mcpd_ctx *ctx, const mcpd_design *design, const uint8_t *y,
     ALLOC(d_Tnu, t.Tnu.size());
     ALLOC(d_init, t.init_pairs.size());
     {
-        const mcpd::ChunkShape cs = mcpd::chunk_shape(t.P, pl->grid, warps, 32 * mcpd::kBankRounds);
+        const mcpd::ChunkShape cs = mcpd::chunk_shape(t.P, pl->grid, warps, mcpd::kBank);
         kp.chunk = cs.chunk;
         kp.bank = std::max(32, cs.chunk);         // a later run may bring more slots
     }

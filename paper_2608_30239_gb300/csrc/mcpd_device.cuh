@@ -64,17 +64,19 @@ static __device__ __forceinline__ void red_add(long long *a, long long v) {
 static __device__ __forceinline__ void red_max(unsigned long long *a, unsigned long long v) {
     asm volatile("red.global.max.u64 [%0], %1;" ::"l"(a), "l"(v) : "memory");
 }
-// W(u) for any lag: sum_{r=k}^{min(l,u)} (floor((u - r) / lag) + 1), through
-// F(n) = sum_{d=0}^{n} floor(d / lag) = lag q (q - 1) / 2 + q (n - q lag + 1), q = floor(n / lag).
-static __device__ __noinline__ long long lag_prefix(long long u, long long k, long long ell, long long lag) {
+// W(u) for any lag: sum_{r=k}^{min(l,u)} (floor((u - r) / lag) + 1) = (m - k + 1) + F(u - k) - F(u - m - 1),
+// m = min(u, l), F(n) = sum_{d=0}^{n} floor(d / lag) = lag q (q - 1) / 2 + q (n - q lag + 1) with
+// q = floor(n / lag).  32-bit divisions (every argument is a step count; with 64-bit ones a pair with
+// lag one sweep spent most of its steps in them), and one of them only beyond l.
+static __device__ __noinline__ long long lag_prefix(uint32_t u, uint32_t k, uint32_t ell, uint32_t lag) {
     if (u < k) return 0;
-    const long long m = u < ell ? u : ell;
-    auto F = [&](long long n) -> long long {
-        if (n < 0) return 0;
-        const long long q = n / lag;
-        return lag * q * (q - 1) / 2 + q * (n - q * lag + 1);
+    const uint32_t m = min(u, ell);
+    auto F = [&](uint32_t n) -> long long {
+        const uint32_t q = n / lag;
+        const unsigned long long lq = static_cast<unsigned long long>(lag) * q;
+        return static_cast<long long>(q ? lq * (q - 1u) / 2u + static_cast<unsigned long long>(q) * (n - lq + 1u) : 0ull);
     };
-    return (m - k + 1) + F(u - k) - F(u - m - 1);
+    return static_cast<long long>(m - k + 1u) + F(u - k) - (u > m ? F(u - m - 1u) : 0ll);
 }
 
 // Add G and G^2 (128-bit, carried into the high word) of one slot to bucket N*_p - 1.

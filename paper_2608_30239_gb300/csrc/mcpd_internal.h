@@ -25,7 +25,7 @@ namespace mcpd {
 constexpr int kRow = 8;              // pool entries per clone row (one 16-byte shared load)
 constexpr int kTSide = kRow + 1;     // acceptance table is kTSide x kTSide, indexed 9 n+ + n-
 constexpr int kMaskDeg = 6;          // uniform degrees up to this use mask-indexed thresholds
-constexpr int kBankRounds = 5;       // a chunk holds at most 32 x this many slots
+constexpr int kBank = 160;           // slots of a chunk, at most
 constexpr int kMaxClones = 65535;
 constexpr int kMaxPools = 1022;      // pool byte offsets must fit 16 bits
 constexpr int kMaxPoolSize = 255;    // per-pool counts are bytes
@@ -53,9 +53,11 @@ enum PairStat {
 #endif
 MCPD_HD inline long long pair_words(long long na, long long W) { return 2 * na + kPairStats + W; }
 // Sampling kernel: an entry is one slot's sums G [na]; a warp's scratch is `bank` entries, the list
-// of those whose pairs are done (two 32-bit words each), and a statistics record per lane.  In 8-byte
-// words.
-MCPD_HD inline long long warp_words(long long bank, long long na) { return bank * na + bank + 32 * kPairStats; }
+// of those whose pairs are done (three 32-bit words each), and a statistics record per lane.  In
+// 8-byte words.
+MCPD_HD inline long long warp_words(long long bank, long long na) {
+    return bank * na + (3 * bank + 1) / 2 + 32 * kPairStats;
+}
 #undef MCPD_HD
 
 // Threads per block the sampling kernel is compiled for.
@@ -215,21 +217,19 @@ inline size_t pairs_smem_bytes(size_t tables, int wpp, int warps) {
     return (tables + static_cast<size_t>(warps) * static_cast<size_t>(wpp) * 128 + 15) / 16 * 16;
 }
 // How `slots` slots are run on `blocks` resident blocks of at most `most` warps: warps per block and
-// slots a warp takes at a time (a chunk).  Slots run for about the same time, so
-//  - more than one round of 32 a warp: the fewest warps that need no more rounds than `most` would,
-//    and chunks of up to kBankRounds rounds (a chunk's pairs fill a warp better, the more slots it has);
-//  - one round: 32 a warp while that keeps kSpreadWarps warps per block busy; below it that many warps
-//    with fewer slots each (a step is shorter, the fewer lanes' branches it carries).
+// slots a warp takes at a time (a chunk).  All of a warp's share at once (in equal parts if a bank
+// cannot hold it): a chunk's single runs are dealt to the lanes one by one, so any number of slots fills
+// them, and its pairs fill a warp the better the more there are.  All warps once the slots give each
+// 16 pairs; below that at most kSpreadWarps per block: 16384 slots with a lag of one sweep, whose time is
+// its pairs', took 37 and 28 ms (two seeds) on 23 warps of 5 slots, 31.5 and 21.7 ms on 12 of 9, 33 and
+// 23 ms on 8 of 14.
 constexpr int kSpreadWarps = 12;
 struct ChunkShape { int warps, chunk; };
 inline ChunkShape chunk_shape(long long slots, long long blocks, int most, long long bank) {
     auto up = [](long long a, long long b) { return (a + b - 1) / b; };
-    const long long rounds = up(slots, blocks * most * 32);
-    const long long fills = up(rounds, std::max<long long>(1, bank / 32)), per = up(rounds, fills);
-    long long w = up(slots, fills * per * blocks * 32);
-    w = std::min<long long>(most, std::max<long long>(w, std::min<long long>(kSpreadWarps, up(slots, blocks))));
+    const long long w = std::min<long long>(most, std::max(up(slots, blocks * 16), std::min<long long>(kSpreadWarps, up(slots, blocks))));
     const long long share = up(slots, blocks * w);
-    return {static_cast<int>(w), static_cast<int>(std::min<long long>(bank, up(share, up(share, bank))))};
+    return {static_cast<int>(w), static_cast<int>(up(share, up(share, bank)))};
 }
 // tables: bytes staged at the start of shared memory (0 for batches); wpp: words per column;
 // P: slots of a single instance (0 = do not shape by rounds); warps: requested warps (0 = auto).

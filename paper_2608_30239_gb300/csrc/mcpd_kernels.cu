@@ -206,7 +206,7 @@ int pairs_shape(int coupled, int scan, int udeg, bool batch, size_t tables, int 
             const int w2 = most(smem_optin / 2);
             int per2 = 1;
             if (w2 >= 1 && resident(w2, &per2) && per2 * w2 > s.per_sm * s.warps) { s.warps = w2; s.per_sm = per2; }
-            if (P > 0) s.warps = chunk_shape(P, static_cast<long long>(sm_count) * s.per_sm, s.warps, 32 * kBankRounds).warps;
+            if (P > 0) s.warps = chunk_shape(P, static_cast<long long>(sm_count) * s.per_sm, s.warps, kBank).warps;
         }
     }
     s.smem = bytes(s.warps);

@@ -79,7 +79,7 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
     const size_t ew = static_cast<size_t>(stride_na);
     auto list = [&]() { return reinterpret_cast<uint32_t *>(wbase + bank * ew); };
     auto pst = [&]() {
-        return reinterpret_cast<unsigned long long *>(wbase + bank * ew + bank + lane * kPairStats);
+        return reinterpret_cast<unsigned long long *>(wbase + bank * ew + (3 * bank + 1) / 2 + lane * kPairStats);
     };
     unsigned long long *const counters = BATCH ? bp.counters : p.counters;
 #pragma unroll
@@ -170,7 +170,7 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
     bool dirty = false;                   // some bit of its column may be set
     bool undo = false;                    // a doomed replication run again to take its events back
     bool plus = false;                    // a bit that turns 0 adds its event's weight (X; Y the other way)
-    uint32_t slot_local = 0, slot_g = 0, r = 0, t = 0, S = 0, N = 0, D = 0, stop = 0;
+    uint32_t slot_local = 0, slot_g = 0, r = 0, t = 0, S = 0, N = 0, D = 0, stop = 0, item = 0;
     long long *sum = nullptr;             // its entry: the slot's sums
     int32_t *trec = nullptr;              // TRACE: the record of the current replication
     uint32_t trace_from = 0;              // TRACE: the single run records from its pair's meeting on
@@ -424,8 +424,34 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
                 cnt = static_cast<uint32_t>(min(per, P - static_cast<long long>(first)));
             }
         }
-        uint32_t head = 0, ready = 0;     // single runs: entries taken, entries whose pairs are done
+        // Single runs, the chunk's (slot, replication) pairs: any lane takes any of them, for a
+        // slot's sums take reductions from every lane.  The list holds, per slot whose pairs are done,
+        // its entry, N and how many of its N runs are left (the last one flushes the entry); head and
+        // hr are the next run's.
+        uint32_t head = 0, hr = 0, ready = 0;
         role = 0; on = false;
+        auto assign_runs = [&]() -> bool {
+            bool got = false;
+            while (head < ready) {
+                const unsigned idle = __ballot_sync(FULL, role == 0);
+                if (!idle) break;
+                const uint32_t n = __ldcg(list() + 3 * head + 1);
+                const uint32_t k = min(n - hr, static_cast<uint32_t>(__popc(idle)));
+                const uint32_t rank = __popc(idle & ((1u << lane) - 1u));
+                if (role == 0 && rank < k) {
+                    take(__ldcg(list() + 3 * head));
+                    N = n;
+                    r = hr + rank;
+                    item = head;
+                    role = 1;
+                    got = true;
+                }
+                hr += k;
+                if (hr == n) { ++head; hr = 0; }
+            }
+            return got;
+        };
+        auto last_run = [&]() -> bool { return atomicSub(list() + 3 * item + 2, 1u) == 1u; };
 
         // ---- Phase 1: pairs to their meetings, and single runs on the lanes that are left over.
         if constexpr (COUPLED) {
@@ -461,7 +487,7 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
                                 const uint32_t a = m - ws0 + 1u;
                                 long long w = static_cast<long long>((static_cast<unsigned long long>(a) * (single ? 2u : a + 1u)) >> 1) +
                                               static_cast<long long>(static_cast<unsigned long long>(single ? 0u : u - m) * wcap);
-                                if (lag != 1u && !single) w = lag_prefix(u, v_k(), ell, lag);
+                                if (lag != 1u && !single) w = lag_prefix(u, ws0, ell, lag);
                                 red_add(sum + s.I, (s.z != 0) == plus ? w : -w);
                             }
                         }
@@ -493,12 +519,13 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
                 if (begin || __any_sync(FULL, ended)) {
                     begin = false;
                     __syncwarp();         // the columns as every lane's steps left them
-                    bool restart = false, drop = false, done = false, banked = false;
+                    bool restart = false, out = false, done = false, banked = false;
                     uint32_t close = 0;
                     if (ended) {
                         if (role == 1) {
                             close = wstep(ell);
-                            if (++r < N) restart = true; else done = true;
+                            out = last_run();
+                            done = true;
                         } else {
                             // 1 completed (met, or unmet at the meeting cap), 2 doomed (it cannot end
                             // within B), 3 step limit
@@ -516,7 +543,7 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
                             bool over = false;             // the slot ends here
                             if (how == 1) {
                                 if (capped && role == 2) {     // the open intervals of X_c and Y_{c-L}
-                                    const long long wc = t < lag ? 0ll : lag_prefix(t - lag, v_k(), ell, lag);
+                                    const long long wc = t < lag ? 0ll : lag_prefix(t - lag, ws0, ell, lag);
                                     for (uint32_t q = 0; q < W && wc != 0; ++q) {
                                         const uint32_t xw = st[q * 32];
                                         uint32_t dm = xw ^ st[q * 32 + 16];
@@ -545,7 +572,7 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
                                 else over = true;
                             } else {
                                 over = true;
-                                drop = role == 2;
+                                out = role == 2;           // the slot is dropped
                             }
                             if (over) {
                                 if (role == 2) {
@@ -587,13 +614,13 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
                         if (m) {
                             if (banked) {
                                 const uint32_t at = ready + __popc(m & ((1u << lane) - 1u));
-                                list()[2 * at] = slot_local - first;
-                                list()[2 * at + 1] = N;
+                                list()[3 * at] = slot_local - first;
+                                list()[3 * at + 1] = N;
+                                list()[3 * at + 2] = N;
                             }
                             ready += __popc(m);
                             __syncwarp();
                         }
-                        const bool out = drop || (done && role == 1);
                         if (__any_sync(FULL, out)) flush(out, role == 1 ? N : 0u);
                         if (done) role = 0;
                     }
@@ -611,22 +638,10 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
                         }
                         taken = min(cnt, taken + __popc(pairs));
                     }
-                    if (taken == cnt && head < ready) {
-                        const unsigned idle = __ballot_sync(FULL, role == 0);
-                        const uint32_t at = head + __popc(idle & ((1u << lane) - 1u));
-                        if (role == 0 && at < ready) {
-                            take(__ldcg(list() + 2 * at));
-                            N = __ldcg(list() + 2 * at + 1);
-                            role = 1;
-                            restart = true;
-                        }
-                        head = min(ready, head + __popc(idle));
-                    }
-                    // Once no pair is left, single runs wait at a replication's end for Phase 2.
                     pm = __ballot_sync(FULL, role >= 2);
-                    const bool go = restart && (role >= 2 || (pm != 0 && ell > 0));
-                    start_random(go);
-                    if (go) {
+                    if (taken == cnt && pm != 0 && ell > 0 && assign_runs()) restart = true;
+                    start_random(restart);
+                    if (restart) {
                         t = 0;
                         // Only a pair's Hamming distance comes to 0: a single run stops at l, and
                         // so does a pair if its step limit lies below l (it runs into the limit).
@@ -657,33 +672,26 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
                 }
             }
         } else {
+            const uint32_t B = v_B(), n = max(1u, B / ell);      // ell: a chain's b + T - 1 >= 1 steps
+            for (uint32_t idx = lane; idx < cnt; idx += 32) {
+                take(idx);
+                list()[3 * idx] = idx;
+                list()[3 * idx + 1] = n;
+                list()[3 * idx + 2] = n;
+                stat_add(kPsProgress, static_cast<unsigned long long>(n) * ell);
+                stat_add(kPsSiteUpdates, static_cast<unsigned long long>(n) * ell);
+                stat_add(kPsStarted, n);
+                stat_add(kPsRetained, n);
+                if (ell > B) stat_add(kPsZero, 1);
+                record_slot(n, static_cast<long long>(n) * ell, n);
+            }
             ready = cnt;
+            __syncwarp();
         }
 
         // ---- Phase 2: single runs, all lanes in step.
         for (;;) {
-            if (head < ready) {
-                const unsigned idle = __ballot_sync(FULL, role == 0);
-                const uint32_t at = head + __popc(idle & ((1u << lane) - 1u));
-                if (role == 0 && at < ready) {
-                    if constexpr (COUPLED) {
-                        take(__ldcg(list() + 2 * at));
-                        N = __ldcg(list() + 2 * at + 1);
-                    } else {
-                        take(at);
-                        const uint32_t B = v_B();
-                        N = max(1u, B / ell);            // l = b + T - 1 >= 1 steps each
-                        stat_add(kPsProgress, static_cast<unsigned long long>(N) * ell);
-                        stat_add(kPsSiteUpdates, static_cast<unsigned long long>(N) * ell);
-                        stat_add(kPsStarted, N);
-                        stat_add(kPsRetained, N);
-                        if (ell > B) stat_add(kPsZero, 1);
-                        record_slot(N, static_cast<long long>(N) * ell, N);
-                    }
-                    role = 1;
-                }
-                head = min(ready, head + __popc(idle));
-            }
+            assign_runs();
             if (!__any_sync(FULL, role == 1)) break;
             start_random(role == 1);
             if (role == 1) {
@@ -776,12 +784,11 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
                     trec[2] = 1;
                     trec[3] = static_cast<int32_t>(r);
                 }
-                ++r;
             }
             __syncwarp();
-            const bool out = role == 1 && r >= N;
+            const bool out = role == 1 && last_run();
             if (__any_sync(FULL, out)) flush(out, N);
-            if (out) role = 0;
+            role = 0;
         }
     }
 
