@@ -47,7 +47,7 @@ struct mcpd_plan {
     long long last_pairs = 0;        // pairs the last launch held (its grid x block)
     mutable int64_t h2d_bytes = 0, d2h_bytes = 0;   // bytes copied between host and device (fetches too)
     size_t scratch_words() const {
-        return static_cast<size_t>(grid) * (block / 32) * mcpd::warp_words(kp.bank, t.na);
+        return static_cast<size_t>(grid) * (block / 32) * mcpd::warp_words(kp.bank, t.na, t.coupled);
     }
 };
 
@@ -708,7 +708,7 @@ int batch_shape(mcpd_ctx *ctx, mcpd_batch *b, int warps, int lanes = 1) {
             c.grid = static_cast<int>(std::max<long long>(1, std::min<long long>(static_cast<long long>(ctx->sm_count) * per_sm,
                                                                                   (units + w - 1) / w)));
             c.pairs = static_cast<long long>(c.grid) * w * std::min(32, c.bp.bank);
-            c.scratch_words = static_cast<size_t>(c.grid) * w * mcpd::warp_words(c.bp.bank, c.bp.max_na);
+            c.scratch_words = static_cast<size_t>(c.grid) * w * mcpd::warp_words(c.bp.bank, c.bp.max_na, b->coupled);
         } else {
             const size_t per_warp = static_cast<size_t>(32 / lanes) * 2 * c.bp.max_wpp * 4;
             const int cap = mcpd::group_max_threads(lanes) / 32;

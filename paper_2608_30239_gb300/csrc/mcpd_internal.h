@@ -53,10 +53,10 @@ enum PairStat {
 #endif
 MCPD_HD inline long long pair_words(long long na, long long W) { return 2 * na + kPairStats + W; }
 // Sampling kernel: an entry is one slot's sums G [na]; a warp's scratch is `bank` entries, the list
-// of those whose pairs are done (three 32-bit words each), and a statistics record per lane.  In
-// 8-byte words.
-MCPD_HD inline long long warp_words(long long bank, long long na) {
-    return bank * na + (3 * bank + 1) / 2 + 32 * kPairStats;
+// of those whose pairs are done (three 32-bit words each), a statistics record per lane and, coupled,
+// sums per pair (at most 16, and one per slot of a chunk).  In 8-byte words.
+MCPD_HD inline long long warp_words(long long bank, long long na, bool coupled) {
+    return bank * na + (3 * bank + 1) / 2 + 32 * kPairStats + (coupled ? (bank < 16 ? bank : 16) * na : 0);
 }
 #undef MCPD_HD
 
@@ -130,7 +130,7 @@ struct KParams {
     const uint64_t *Tnu;
     const uint32_t *init_pairs;       // [n_init_pairs]
     int32_t n_init_pairs;
-    long long *pair_scratch;          // [warps][warp_words(bank, na)]
+    long long *pair_scratch;          // [warps][warp_words(bank, na, coupled)]
     unsigned long long *S1;           // [nb][na]
     unsigned long long *S2lo;         // [nb][na]
     unsigned long long *S2hi;         // [nb][na]
@@ -198,7 +198,7 @@ struct BParams {
     int32_t n_inst, coupled, scan, max_wpp;
     int32_t lanes, max_m;             // lanes per pair (1, 8, 16, 32); largest pool count
     long long total_work, total_units;   // slots; chunks
-    long long *pair_scratch;          // [warps][warp_words(bank, max_na)], or per pair pair_words (lane groups)
+    long long *pair_scratch;          // [warps][warp_words(bank, max_na, coupled)], or per pair pair_words (lane groups)
     unsigned long long *counters;
     int *error;
     int32_t max_na, max_W;

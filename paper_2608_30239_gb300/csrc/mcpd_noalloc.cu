@@ -129,12 +129,12 @@ extern "C" int mcpd_decode_noalloc(mcpd_ctx *ctx, const mcpd_design *design, con
     for (bool first = true;; first = false) {
         chunk = static_cast<int>(std::min<long long>(32, 4 * up(t.P, 4ll * grid * warps)));
         if (first) warps = static_cast<int>(std::min<long long>(warps, up(t.P, static_cast<long long>(grid) * chunk)));
-        if (static_cast<size_t>(grid) * warps * warp_words(chunk, t.na) * 8 <= room || (grid == 1 && warps == 1)) break;
+        if (static_cast<size_t>(grid) * warps * warp_words(chunk, t.na, t.coupled) * 8 <= room || (grid == 1 && warps == 1)) break;
         if (warps > 1) --warps; else --grid;
     }
     const size_t smem = pairs_smem_bytes(tables, t.wpp, warps);
     const size_t all_warps = static_cast<size_t>(grid) * warps;
-    const size_t o_pair = take(all_warps * static_cast<size_t>(warp_words(chunk, t.na)) * 8);
+    const size_t o_pair = take(all_warps * static_cast<size_t>(warp_words(chunk, t.na, t.coupled)) * 8);
     if (off > kNoAllocScratchBytes) return fail(ctx, MCPD_ETOO_LARGE, "no-alloc scratch layout overflow");
 
     unsigned char *b = static_cast<unsigned char *>(base);

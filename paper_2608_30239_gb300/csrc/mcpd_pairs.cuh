@@ -70,17 +70,19 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
     __syncthreads();
 
     // This warp's scratch (see warp_words): `bank` entries (a slot's sums), a list of the entries
-    // whose pairs are done, and a statistics record per lane.
+    // whose pairs are done, a statistics record per lane, and sums per pair.
     const int stride_na = BATCH ? bp.max_na : p.na;
     const int bank = BATCH ? bp.bank : p.bank;
     long long *const wbase = (BATCH ? bp.pair_scratch : p.pair_scratch) +
                              static_cast<size_t>(blockIdx.x * nwarps + warp) *
-                                 static_cast<size_t>(warp_words(bank, stride_na));
+                                 static_cast<size_t>(warp_words(bank, stride_na, COUPLED));
     const size_t ew = static_cast<size_t>(stride_na);
     auto list = [&]() { return reinterpret_cast<uint32_t *>(wbase + bank * ew); };
     auto pst = [&]() {
         return reinterpret_cast<unsigned long long *>(wbase + bank * ew + (3 * bank + 1) / 2 + lane * kPairStats);
     };
+    // Pair i's events of the replication it is running.
+    auto pair_sums = [&](int i) { return wbase + bank * ew + (3 * bank + 1) / 2 + 32 * kPairStats + i * ew; };
     unsigned long long *const counters = BATCH ? bp.counters : p.counters;
 #pragma unroll
     for (int i = 0; i < kPairStats; ++i) pst()[i] = 0ull;
@@ -168,10 +170,9 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
     int role = 0;
     bool on = false;                      // takes steps
     bool dirty = false;                   // some bit of its column may be set
-    bool undo = false;                    // a doomed replication run again to take its events back
-    bool plus = false;                    // a bit that turns 0 adds its event's weight (X; Y the other way)
+    bool events = false;                  // its pair's sums may hold something
     uint32_t slot_local = 0, slot_g = 0, r = 0, t = 0, S = 0, N = 0, D = 0, stop = 0, item = 0;
-    long long *sum = nullptr;             // its entry: the slot's sums
+    long long *sum = nullptr;             // where its events go: the slot's entry, or its pair's sums
     int32_t *trec = nullptr;              // TRACE: the record of the current replication
     uint32_t trace_from = 0;              // TRACE: the single run records from its pair's meeting on
 
@@ -380,10 +381,11 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
     };
     // Point the lane at slot `idx` of the chunk and its entry.
     uint32_t first = 0, cnt = 0;          // the chunk: slots first .. first + cnt - 1
+    auto entry = [&]() { return wbase + static_cast<size_t>(slot_local - first) * ew; };
     auto take = [&](uint32_t idx) {
         slot_local = first + idx;
         slot_g = static_cast<uint32_t>(v_slot_offset() + static_cast<long long>(slot_local));
-        sum = wbase + idx * ew;
+        sum = entry();
         r = 0;
     };
 
@@ -488,7 +490,8 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
                                 long long w = static_cast<long long>((static_cast<unsigned long long>(a) * (single ? 2u : a + 1u)) >> 1) +
                                               static_cast<long long>(static_cast<unsigned long long>(single ? 0u : u - m) * wcap);
                                 if (lag != 1u && !single) w = lag_prefix(u, ws0, ell, lag);
-                                red_add(sum + s.I, (s.z != 0) == plus ? w : -w);
+                                red_add(sum + s.I, (s.z != 0) != (role == 3) ? w : -w);
+                                events = true;
                             }
                         }
                     }
@@ -502,7 +505,7 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
                         }
                     }
                     if constexpr (TRACE) {
-                        if (on && !undo) {
+                        if (on) {
                             if (role == 1) trace_step(s.I, t, f, f);
                             else if (role == 2) trace_step(s.I, t, f, (fb >> (lane | 16)) & 1u);
                         }
@@ -519,8 +522,9 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
                 if (begin || __any_sync(FULL, ended)) {
                     begin = false;
                     __syncwarp();         // the columns as every lane's steps left them
-                    bool restart = false, out = false, done = false, banked = false;
+                    bool restart = false, out = false, done = false, banked = false, keep = false;
                     uint32_t close = 0;
+                    const bool pair_ended = ended && role >= 2;
                     if (ended) {
                         if (role == 1) {
                             close = wstep(ell);
@@ -534,14 +538,15 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
                             const bool capped = !met && v_capped() && t >= v_step_limit();
                             const int how = met || capped ? 1 : ((r > 0 && t >= B - S) ? 2 : 3);
                             const uint32_t C = met ? max(ell, t) : t, tau = met ? t : 0u;
-                            if (TRACE && trec && role == 2 && !undo) {
+                            if (TRACE && trec && role == 2) {
                                 trec[0] = static_cast<int32_t>(tau);
                                 trec[1] = static_cast<int32_t>(C);
                                 trec[2] = how;
                                 trec[3] = static_cast<int32_t>(r);
                             }
                             bool over = false;             // the slot ends here
-                            if (how == 1) {
+                            keep = how == 1;
+                            if (keep) {
                                 if (capped && role == 2) {     // the open intervals of X_c and Y_{c-L}
                                     const long long wc = t < lag ? 0ll : lag_prefix(t - lag, ws0, ell, lag);
                                     for (uint32_t q = 0; q < W && wc != 0; ++q) {
@@ -551,7 +556,7 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
                                         while (dm) {
                                             const int b = __ffs(dm) - 1;
                                             dm &= dm - 1;
-                                            red_add(sum + q * 32 + b, ((xw >> b) & 1u) ? wc : -wc);
+                                            red_add(entry() + q * 32 + b, ((xw >> b) & 1u) ? wc : -wc);
                                         }
                                     }
                                 }
@@ -565,14 +570,9 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
                                     if (S > B) stat_add(kPsZero, 1);   // only a slot's first replication ends beyond B
                                 }
                                 if (S < B && B - S >= v_unit()) { ++r; restart = true; } else over = true;
-                            } else if (how == 2) {
-                                // its events (from t - L = k on) leave the slot: the same draws
-                                // once more, with the opposite signs
-                                if (!undo && t > lag && t - lag > ws0) { undo = true; restart = true; }
-                                else over = true;
                             } else {
                                 over = true;
-                                out = role == 2;           // the slot is dropped
+                                out = how == 3 && role == 2;      // the slot is dropped
                             }
                             if (over) {
                                 if (role == 2) {
@@ -591,10 +591,42 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
                                     record_slot(how == 3 ? 0u : N, static_cast<long long>(S), r + 1);
                                     banked = how != 3;
                                 }
-                                undo = false;
                                 done = true;
                             }
                         }
+                    }
+                    // A retained replication's events join its slot's sums; those of a doomed one, or of
+                    // a pair at its step limit, go.  Coalesced, by the whole warp; pairs that met before
+                    // the window have none.
+                    {
+                        unsigned m = __ballot_sync(FULL, pair_ended && events);
+                        m = (m | m >> 16) & 0xFFFFu;
+                        if (m) {
+                            __threadfence();
+                            __syncwarp();
+                            while (m) {
+                                const int src = __ffs(m) - 1;
+                                m &= m - 1;
+                                const bool keep_s = __shfl_sync(FULL, keep ? 1 : 0, src) != 0;
+                                long long *const to = wbase + static_cast<size_t>(__shfl_sync(FULL, slot_local, src) - first) * ew;
+                                long long *const from = pair_sums(src);
+                                for (int j0 = lane; j0 < na; j0 += 128) {
+                                    long long g[4];
+#pragma unroll
+                                    for (int u = 0; u < 4; ++u) g[u] = j0 + 32 * u < na ? __ldcg(from + j0 + 32 * u) : 0;
+#pragma unroll
+                                    for (int u = 0; u < 4; ++u)
+                                        if (g[u] != 0) {
+                                            from[j0 + 32 * u] = 0;
+                                            if (keep_s) red_add(to + j0 + 32 * u, g[u]);
+                                        }
+                                }
+                            }
+                            __threadfence();
+                            __syncwarp();
+                            if (pair_ended) events = false;
+                        }
+                        if (pair_ended && done) sum = entry();
                     }
                     // columns of the ended lanes (a lane that never flipped has an empty one)
                     {
@@ -633,6 +665,7 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
                         if (((pairs >> me) & 1u) && at < cnt) {
                             role = lane < 16 ? 2 : 3;
                             take(at);
+                            sum = pair_sums(lane & 15);
                             S = 0; N = 0;
                             restart = true;
                         }
@@ -647,7 +680,6 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
                         // so does a pair if its step limit lies below l (it runs into the limit).
                         D = role == 1 || !quick ? 0x40000000u : 0u;
                         still = role == 3 ? lag : 0u;
-                        plus = (role != 3) != undo;
                         stop = role == 1 ? ell : min(r > 0 ? v_B() - S : 0xFFFFFFFFu, v_step_limit());
                         trace_at();
                         on = true;
