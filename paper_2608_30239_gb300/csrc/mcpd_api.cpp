@@ -40,8 +40,9 @@ struct mcpd_plan {
     bool dirty = true;
     bool ran = false;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
-    std::vector<void *> allocs;
-    double *est_dev = nullptr, *se_dev = nullptr;    // used by mcpd_decode
+    void *mem = nullptr;             // all of the plan's device memory
+    size_t clear_bytes = 0, stat_bytes = 0;   // S1 .. error, of which the last stat_bytes are counters and error
+    double *est_dev = nullptr, *se_dev = nullptr;    // used by mcpd_decode (se_dev follows est_dev)
     int64_t n_trace = 0;
     int64_t slots_run = 0;           // slots in the buckets since the last run that cleared them
     long long last_pairs = 0;        // pairs the last launch held (its grid x block)
@@ -76,17 +77,6 @@ int cu_status(mcpd_ctx *ctx, cudaError_t e, const char *what) {
         const int r_ = cu_status(ctx, (call), #call);                                         \
         if (r_ != MCPD_OK) { cleanup; return r_; }                                            \
     } while (0)
-
-template <typename T>
-int dev_alloc(mcpd_ctx *ctx, mcpd_plan *pl, T **ptr, size_t count) {
-    *ptr = nullptr;
-    if (count == 0) return MCPD_OK;
-    void *p = nullptr;
-    CU(cudaMalloc(&p, count * sizeof(T)));
-    pl->allocs.push_back(p);
-    *ptr = static_cast<T *>(p);
-    return MCPD_OK;
-}
 
 }  // namespace
 
@@ -221,14 +211,22 @@ int mcpd_ctx_create(int device, void *cuda_stream, mcpd_ctx **out) {
     return MCPD_OK;
 }
 
-void mcpd_ctx_destroy(mcpd_ctx *ctx) { delete ctx; }
+void mcpd_ctx_destroy(mcpd_ctx *ctx) {
+    if (!ctx) return;
+    if (ctx->stage_bytes) {
+        cudaSetDevice(ctx->device);
+        cudaFreeHost(ctx->stage_host);
+        cudaFree(ctx->stage_dev);
+    }
+    delete ctx;
+}
 
 const char *mcpd_last_error(const mcpd_ctx *ctx) { return ctx ? ctx->err.c_str() : "null context"; }
 
 void mcpd_plan_destroy(mcpd_plan *pl) {
     if (!pl) return;
     if (pl->device >= 0) cudaSetDevice(pl->device);
-    for (void *p : pl->allocs) cudaFree(p);
+    cudaFree(pl->mem);
     if (pl->ev0) cudaEventDestroy(pl->ev0);
     if (pl->ev1) cudaEventDestroy(pl->ev1);
     delete pl;
@@ -264,57 +262,72 @@ int mcpd_plan_create(mcpd_ctx *ctx, const mcpd_design *design, const uint8_t *y,
     pl->grid = ctx->sm_count * shape.per_sm;
     pl->pairs = static_cast<long long>(pl->grid) * pl->block;
 
+    // One device allocation: the tables (uploaded in one copy), what a run clears (one memset), the
+    // outputs of mcpd_decode, records and traces, the kernel's scratch.  (Fourteen allocations, five
+    // copies and the launch permission of every kernel build made a plan of a 20-clone problem cost 333 us.)
     mcpd::KParams &kp = pl->kp;
-    uint64_t *d_alias = nullptr, *d_T = nullptr, *d_Tnu = nullptr;
-    uint16_t *d_rows = nullptr;
-    uint32_t *d_init = nullptr;
-#define ALLOC(ptr, n)                                                        \
-    do {                                                                     \
-        int r_ = dev_alloc(ctx, pl, &(ptr), (n));                            \
-        if (r_ != MCPD_OK) { mcpd_plan_destroy(pl); return r_; }             \
-    } while (0)
-    ALLOC(d_alias, t.alias.size());
-    ALLOC(d_rows, mcpd::kernel_rows(t).size());
-    ALLOC(d_T, mcpd::kernel_T(t).size());
-    ALLOC(d_Tnu, t.Tnu.size());
-    ALLOC(d_init, t.init_pairs.size());
     {
         const mcpd::ChunkShape cs = mcpd::chunk_shape(t.P, pl->grid, warps, mcpd::kBank);
         kp.chunk = cs.chunk;
         kp.bank = std::max(32, cs.chunk);         // a later run may bring more slots
     }
-    ALLOC(kp.pair_scratch, pl->scratch_words());
-    ALLOC(kp.S1, static_cast<size_t>(t.nb) * t.na);
-    ALLOC(kp.S2lo, static_cast<size_t>(t.nb) * t.na);
-    ALLOC(kp.S2hi, static_cast<size_t>(t.nb) * t.na);
-    ALLOC(kp.bcount, static_cast<size_t>(t.nb));
-    ALLOC(kp.counters, static_cast<size_t>(mcpd::kNumCounters));
-    ALLOC(kp.error, 1);
-    ALLOC(pl->est_dev, static_cast<size_t>(t.na));
-    ALLOC(pl->se_dev, static_cast<size_t>(t.na));
+    if (t.trace_stride > 0) pl->n_trace = (t.P + t.trace_stride - 1) / t.trace_stride;
+    size_t total = 0;
+    auto take = [&](size_t bytes, size_t align) {
+        total = (total + align - 1) / align * align;
+        const size_t at = total;
+        total += bytes;
+        return at;
+    };
+    const size_t nbna = static_cast<size_t>(t.nb) * t.na;
+    const size_t o_alias = take(t.alias.size() * 8, 16), o_rows = take(mcpd::kernel_rows(t).size() * 2, 16);
+    const size_t o_T = take(mcpd::kernel_T(t).size() * 8, 16), o_Tnu = take(t.Tnu.size() * 8, 16);
+    const size_t o_init = take(t.init_pairs.size() * 4, 16), tables_end = total;
+    const size_t o_S = take(nbna * 3 * 8, 256), o_bcount = take(static_cast<size_t>(t.nb) * 8, 8);
+    const size_t o_counters = take(mcpd::kNumCounters * 8, 8), o_error = take(8, 8);
+    pl->clear_bytes = total - o_S;
+    pl->stat_bytes = total - o_counters;
+    const size_t o_est = take(static_cast<size_t>(t.na) * 2 * 8, 256);
+    const size_t slots = t.record_slots ? static_cast<size_t>(t.P) : 0;
+    const size_t o_nstar = take(slots * 4, 256), o_slot_S = take(slots * 8, 256), o_reps = take(slots * 4, 256);
+    const size_t o_trace = take(static_cast<size_t>(pl->n_trace) * t.na * 8, 256);
+    const size_t o_rec = take(static_cast<size_t>(pl->n_trace) * t.trace_reps * (4 + t.trace_steps) * 4, 256);
+    const size_t o_scratch = take(pl->scratch_words() * 8, 256);
+    CU_OR(cudaMalloc(&pl->mem, total), mcpd_plan_destroy(pl));
+    unsigned char *const mem = static_cast<unsigned char *>(pl->mem);
+    std::vector<unsigned char> tab(tables_end);
+    auto put = [&](size_t at, const void *src, size_t bytes) { if (bytes) std::memcpy(tab.data() + at, src, bytes); };
+    put(o_alias, t.alias.data(), t.alias.size() * 8);
+    put(o_rows, mcpd::kernel_rows(t).data(), mcpd::kernel_rows(t).size() * 2);
+    put(o_T, mcpd::kernel_T(t).data(), mcpd::kernel_T(t).size() * 8);
+    put(o_Tnu, t.Tnu.data(), t.Tnu.size() * 8);
+    put(o_init, t.init_pairs.data(), t.init_pairs.size() * 4);
+    CU_OR(cudaMemcpyAsync(mem, tab.data(), tables_end, cudaMemcpyHostToDevice, ctx->stream), mcpd_plan_destroy(pl));
+    pl->h2d_bytes += static_cast<int64_t>(tables_end);
+    kp.alias = reinterpret_cast<const uint64_t *>(mem + o_alias);
+    kp.rows = reinterpret_cast<const uint16_t *>(mem + o_rows);
+    kp.T = reinterpret_cast<const uint64_t *>(mem + o_T);
+    kp.Tnu = t.Tnu.empty() ? nullptr : reinterpret_cast<const uint64_t *>(mem + o_Tnu);
+    kp.init_pairs = reinterpret_cast<const uint32_t *>(mem + o_init);
+    kp.n_init_pairs = static_cast<int32_t>(t.init_pairs.size());
+    kp.S1 = reinterpret_cast<unsigned long long *>(mem + o_S);
+    kp.S2lo = kp.S1 + nbna;
+    kp.S2hi = kp.S2lo + nbna;
+    kp.bcount = reinterpret_cast<unsigned long long *>(mem + o_bcount);
+    kp.counters = reinterpret_cast<unsigned long long *>(mem + o_counters);
+    kp.error = reinterpret_cast<int *>(mem + o_error);
+    pl->est_dev = reinterpret_cast<double *>(mem + o_est);
+    pl->se_dev = pl->est_dev + t.na;
     if (t.record_slots) {
-        ALLOC(kp.slot_nstar, static_cast<size_t>(t.P));
-        ALLOC(kp.slot_S, static_cast<size_t>(t.P));
-        ALLOC(kp.slot_reps, static_cast<size_t>(t.P));
+        kp.slot_nstar = reinterpret_cast<int32_t *>(mem + o_nstar);
+        kp.slot_S = reinterpret_cast<long long *>(mem + o_slot_S);
+        kp.slot_reps = reinterpret_cast<int32_t *>(mem + o_reps);
     }
     if (t.trace_stride > 0) {
-        pl->n_trace = (t.P + t.trace_stride - 1) / t.trace_stride;
-        ALLOC(kp.trace_G, static_cast<size_t>(pl->n_trace) * t.na);
-        if (t.trace_steps > 0)
-            ALLOC(kp.trace_rec, static_cast<size_t>(pl->n_trace) * t.trace_reps * (4 + t.trace_steps));
+        kp.trace_G = reinterpret_cast<long long *>(mem + o_trace);
+        if (t.trace_steps > 0) kp.trace_rec = reinterpret_cast<int32_t *>(mem + o_rec);
     }
-#undef ALLOC
-    CU_OR(cudaMemcpyAsync(d_alias, t.alias.data(), t.alias.size() * 8, cudaMemcpyHostToDevice, ctx->stream), mcpd_plan_destroy(pl));
-    CU_OR(cudaMemcpyAsync(d_rows, mcpd::kernel_rows(t).data(), mcpd::kernel_rows(t).size() * 2, cudaMemcpyHostToDevice, ctx->stream), mcpd_plan_destroy(pl));
-    CU_OR(cudaMemcpyAsync(d_T, mcpd::kernel_T(t).data(), mcpd::kernel_T(t).size() * 8, cudaMemcpyHostToDevice, ctx->stream), mcpd_plan_destroy(pl));
-    if (!t.Tnu.empty())
-        CU_OR(cudaMemcpyAsync(d_Tnu, t.Tnu.data(), t.Tnu.size() * 8, cudaMemcpyHostToDevice, ctx->stream), mcpd_plan_destroy(pl));
-    if (!t.init_pairs.empty())
-        CU_OR(cudaMemcpyAsync(d_init, t.init_pairs.data(), t.init_pairs.size() * 4, cudaMemcpyHostToDevice, ctx->stream), mcpd_plan_destroy(pl));
-    pl->h2d_bytes += static_cast<int64_t>(t.alias.size() * 8 + mcpd::kernel_rows(t).size() * 2 +
-                                          mcpd::kernel_T(t).size() * 8 + t.Tnu.size() * 8 + t.init_pairs.size() * 4);
-    kp.alias = d_alias; kp.rows = d_rows; kp.T = d_T; kp.Tnu = t.Tnu.empty() ? nullptr : d_Tnu;
-    kp.init_pairs = d_init; kp.n_init_pairs = static_cast<int32_t>(t.init_pairs.size());
+    kp.pair_scratch = reinterpret_cast<long long *>(mem + o_scratch);
     kp.na = t.na; kp.m = t.m; kp.W = t.W; kp.Mp = t.Mp; kp.wpp = t.wpp; kp.deg = t.deg_max; kp.udeg = t.udeg;
     kp.nb = static_cast<int32_t>(t.nb); kp.scan = t.scan;
     kp.dummy_entry = t.dummy_entry; kp.dummy_word = t.dummy_word;
@@ -380,15 +393,9 @@ int run_range(mcpd_ctx *ctx, mcpd_plan *pl, int64_t slots, bool accumulate, doub
     kp.warps = warps;
     kp.chunk = cs.chunk;
     const size_t smem = mcpd::pairs_smem_bytes(kp.smem_tables, t.wpp, warps);
-    const size_t nbna = static_cast<size_t>(t.nb) * t.na;
-    if (!accumulate) {
-        CU(cudaMemsetAsync(kp.S1, 0, nbna * 8, ctx->stream));
-        CU(cudaMemsetAsync(kp.S2lo, 0, nbna * 8, ctx->stream));
-        CU(cudaMemsetAsync(kp.S2hi, 0, nbna * 8, ctx->stream));
-        CU(cudaMemsetAsync(kp.bcount, 0, static_cast<size_t>(t.nb) * 8, ctx->stream));
-    }
-    CU(cudaMemsetAsync(kp.counters, 0, mcpd::kNumCounters * 8, ctx->stream));
-    CU(cudaMemsetAsync(kp.error, 0, sizeof(int), ctx->stream));
+    // the buckets, their counts, the counters and the error flag; or, extending, the last two only
+    if (accumulate) CU(cudaMemsetAsync(kp.counters, 0, pl->stat_bytes, ctx->stream));
+    else CU(cudaMemsetAsync(kp.S1, 0, pl->clear_bytes, ctx->stream));
     if (pl->dirty) {   // the kernel leaves these zeroed when it completes normally
         CU(cudaMemsetAsync(kp.pair_scratch, 0, pl->scratch_words() * 8, ctx->stream));
     }
@@ -436,12 +443,11 @@ int mcpd_collect(mcpd_ctx *ctx, mcpd_plan *pl, mcpd_stats *stats) {
     if (!ctx || !pl) return MCPD_EINVAL;
     if (!pl->ran) return set_err(ctx, MCPD_EINVAL, "no run to collect");
     CU(cudaSetDevice(ctx->device));
-    unsigned long long c[mcpd::kNumCounters];
-    int error = 0;
+    unsigned long long c[mcpd::kNumCounters + 1];               // the counters, then the error flag
     CU(cudaMemcpyAsync(c, pl->kp.counters, sizeof(c), cudaMemcpyDeviceToHost, ctx->stream));
-    CU(cudaMemcpyAsync(&error, pl->kp.error, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
-    pl->d2h_bytes += static_cast<int64_t>(sizeof(c) + sizeof(int));
+    pl->d2h_bytes += static_cast<int64_t>(sizeof(c));
     CU(cudaStreamSynchronize(ctx->stream));
+    const bool error = static_cast<uint32_t>(c[mcpd::kNumCounters]) != 0;
     float ms = 0.f;
     CU(cudaEventElapsedTime(&ms, pl->ev0, pl->ev1));
     if (stats) {
@@ -510,18 +516,17 @@ int mcpd_decode(mcpd_ctx *ctx, const mcpd_design *design, const uint8_t *y,
     if (rc == MCPD_OK) rc = mcpd_collect(ctx, pl, stats);
     if (rc == MCPD_OK || rc == MCPD_ESTEP_LIMIT) {
         const int32_t na = pl->t.na;
-        std::vector<double> e(na), s(na);
-        cudaError_t c1 = cudaMemcpyAsync(e.data(), pl->est_dev, na * 8, cudaMemcpyDeviceToHost, ctx->stream);
-        cudaError_t c2 = cudaMemcpyAsync(s.data(), pl->se_dev, na * 8, cudaMemcpyDeviceToHost, ctx->stream);
-        cudaError_t c3 = cudaStreamSynchronize(ctx->stream);
-        if (c1 != cudaSuccess || c2 != cudaSuccess || c3 != cudaSuccess) {
+        std::vector<double> es(2 * static_cast<size_t>(na));
+        const cudaError_t c1 = cudaMemcpyAsync(es.data(), pl->est_dev, es.size() * 8, cudaMemcpyDeviceToHost, ctx->stream);
+        const cudaError_t c2 = cudaStreamSynchronize(ctx->stream);
+        if (c1 != cudaSuccess || c2 != cudaSuccess) {
             rc = set_err(ctx, MCPD_ECUDA, "copying results to the host");
         } else {
             if (stats) stats->d2h_bytes += static_cast<int64_t>(2 * na * 8);
             for (int32_t i = 0; i < design->n_clones; ++i) { est[i] = 0.0; se[i] = 0.0; if (active) active[i] = 0; }
             for (int32_t a = 0; a < na; ++a) {
                 const int32_t i = pl->t.active[a];
-                est[i] = e[a]; se[i] = s[a];
+                est[i] = es[a]; se[i] = es[static_cast<size_t>(na) + a];
                 if (active) active[i] = 1;
             }
         }

@@ -18,9 +18,15 @@ struct mcpd_ctx {
     int sm_count = 0;
     size_t smem_optin = 0;
     std::string err;
+    // Staging of mcpd_features_batch, kept between calls up to kKeepStaging bytes: pinned host memory
+    // and device memory of the same size.
+    void *stage_host = nullptr, *stage_dev = nullptr;
+    size_t stage_bytes = 0;
 };
 
 namespace mcpd {
+
+constexpr size_t kKeepStaging = size_t(32) << 20;
 
 constexpr int kRow = 8;              // pool entries per clone row (one 16-byte shared load)
 constexpr int kTSide = kRow + 1;     // acceptance table is kTSide x kTSide, indexed 9 n+ + n-
@@ -255,7 +261,6 @@ int launch_finalize_batch(const InstDesc *insts, int n_inst, const int32_t *clon
 int launch_pairs(const KParams &kp, int grid, int block, size_t smem, void *stream);
 // The recording variants (mcpd_trace.cu): launched by launch_pairs when kp.trace_rec is set.
 int launch_pairs_trace(const KParams &kp, int grid, int block, size_t smem, void *stream);
-int set_trace_smem(size_t bytes);
 int launch_finalize(const unsigned long long *S1, const unsigned long long *S2lo,
                     const unsigned long long *S2hi, int na, int nb, long long P, long long L,
                     double *est, double *se, void *stream);

@@ -106,21 +106,6 @@ PairsFn pick(int coupled, int scan, bool batch, int udeg) {
     }
 }
 
-int set_smem(size_t bytes, bool batch) {
-    for (int c = 0; c < 2; ++c)
-        for (int sc : {MCPD_SCAN_SCORE, MCPD_SCAN_SYSTEMATIC}) {
-            if (c && sc == MCPD_SCAN_SYSTEMATIC) continue;
-            for (int ud = 0; ud <= 8; ++ud) {
-                if (ud && (ud < 3 || (!c && ud > kMaskDeg))) continue;
-                if (batch && ud != batch_kernel_degree(c, 0, ud)) continue;
-                if (cudaFuncSetAttribute(pick(c, sc, batch, ud), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(bytes)) != cudaSuccess)
-                    return MCPD_ECUDA;
-            }
-        }
-    return batch ? MCPD_OK : set_trace_smem(bytes);
-}
-
 int max_warps(int coupled, int scan, int udeg, bool batch) {
     cudaFuncAttributes a{};
     if (cudaFuncGetAttributes(&a, pick(coupled, scan, batch, udeg)) != cudaSuccess) return 16;
@@ -192,7 +177,9 @@ int pairs_shape(int coupled, int scan, int udeg, bool batch, size_t tables, int 
     int w1 = most(smem_optin);
     // The attribute is a permission shared by every launch of the kernel (the classes of a batch
     // have different sizes): allow the device's opt-in maximum.
-    if (set_smem(smem_optin, batch) != MCPD_OK) return MCPD_ECUDA;
+    if (cudaFuncSetAttribute(pick(coupled, scan, batch, udeg), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             static_cast<int>(smem_optin)) != cudaSuccess)
+        return MCPD_ECUDA;
     PairsShape s;
     if (warps > 0) {
         if (warps > w1) return MCPD_EINVAL;

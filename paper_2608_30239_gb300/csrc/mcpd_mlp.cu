@@ -12,6 +12,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstring>
 #include <string>
 #include <vector>
 
@@ -338,75 +339,85 @@ __global__ void mlp_heads_kernel(const long long *seg, const float *Out, double 
     }
 }
 
-// Features, pass 1 (per clone): degree, positive pools, all-positive flag; pool sizes.
-__global__ void feat_pass1(long long n, const int32_t *ptr, const int32_t *pools, const uint8_t *y,
-                           const int64_t *clone_pool_base, int32_t *deg, int32_t *npos,
-                           int32_t *allpos, int32_t *psize, int32_t *nap, const int32_t *clone_inst) {
-    const long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const long long base = clone_pool_base[i];
-    int d = 0, p = 0;
-    for (int e = ptr[i]; e < ptr[i + 1]; ++e) {
-        const long long j = base + pools[e];
-        p += y[j];
-        ++d;
-        atomicAdd(&psize[j], 1);
+// Features.  The designs lie one after the other as the caller holds them: instance s's clone_ptr at
+// ptr + clone_off[s] + s (local offsets), its entries from pools + entry_off[s], its pools from
+// pool_off[s] on.
+struct FeatIn {
+    const int32_t *ptr, *pools;
+    const uint8_t *y;
+    const long long *clone_off, *entry_off, *pool_off;   // [n_inst + 1]
+    const double *consts;                                 // [n_inst][4]: lambda, a+, a-, mean pool size
+    int n_inst;
+    int32_t *psize, *ap_pool, *nap;                       // pool sizes, all-positive clones per pool and per instance
+};
+struct FeatClone { int s; const int32_t *row; int d; long long base; };
+// Clone i: its instance (binary search), its pools, the first pool of its instance.
+__device__ __forceinline__ FeatClone feat_clone(const FeatIn &in, long long i) {
+    int lo = 0, hi = in.n_inst - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (in.clone_off[mid] <= i) lo = mid; else hi = mid - 1;
     }
-    deg[i] = d;
-    npos[i] = p;
-    const int ap = (d > 0 && p == d) ? 1 : 0;
-    allpos[i] = ap;
-    if (ap) atomicAdd(&nap[clone_inst[i]], 1);
+    const int32_t *p = in.ptr + i + lo;
+    const int32_t e0 = p[0] - in.ptr[in.clone_off[lo] + lo];
+    return {lo, in.pools + in.entry_off[lo] + e0, p[1] - p[0], in.pool_off[lo]};
+}
+__device__ __forceinline__ int feat_positive(const FeatIn &in, const FeatClone &c) {
+    int p = 0;
+    for (int e = 0; e < c.d; ++e) p += in.y[c.base + c.row[e]] ? 1 : 0;
+    return p;
 }
 
-__global__ void feat_pass2(long long n, const int32_t *ptr, const int32_t *pools,
-                           const int64_t *clone_pool_base, const int32_t *allpos, int32_t *ap_pool) {
-    const long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (i >= n || !allpos[i]) return;
-    for (int e = ptr[i]; e < ptr[i + 1]; ++e) atomicAdd(&ap_pool[clone_pool_base[i] + pools[e]], 1);
-}
-
-__global__ void feat_pass3(long long n, const int32_t *ptr, const int32_t *pools, const uint8_t *y,
-                           const int64_t *clone_pool_base, const int32_t *deg, const int32_t *npos,
-                           const int32_t *allpos, const int32_t *psize, const int32_t *ap_pool,
-                           const int32_t *nap, const int32_t *clone_inst, const double *consts,
-                           float *Fout) {
+// Pool sizes; per pool and per instance the clones all of whose pools are positive.
+__global__ void feat_counts(long long n, const FeatIn in) {
     const long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    const int s = clone_inst[i];
-    const double lam = consts[4 * s], a_pos = consts[4 * s + 1], a_neg = consts[4 * s + 2], dbar = consts[4 * s + 3];
-    const long long base = clone_pool_base[i];
-    const int d = deg[i], p = npos[i], nn = d - p, ap = allpos[i];
+    const FeatClone c = feat_clone(in, i);
+    const bool all = c.d > 0 && feat_positive(in, c) == c.d;
+    for (int e = 0; e < c.d; ++e) {
+        atomicAdd(&in.psize[c.base + c.row[e]], 1);
+        if (all) atomicAdd(&in.ap_pool[c.base + c.row[e]], 1);
+    }
+    if (all) atomicAdd(&in.nap[c.s], 1);
+}
+
+__global__ void feat_rows(long long n, const FeatIn in, float *Fout) {
+    const long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const FeatClone c = feat_clone(in, i);
+    const double lam = in.consts[4 * c.s], a_pos = in.consts[4 * c.s + 1], a_neg = in.consts[4 * c.s + 2], dbar = in.consts[4 * c.s + 3];
+    const int d = c.d, p = feat_positive(in, c), nn = d - p, ap = d > 0 && p == d ? 1 : 0;
     double sum_d = 0.0, sum_dpos = 0.0, sum_inv = 0.0;
     int min_ap = 1 << 30, sole = 0, unexplained = 0;
-    for (int e = ptr[i]; e < ptr[i + 1]; ++e) {
-        const long long j = base + pools[e];
-        sum_d += psize[j];
-        if (y[j]) {
-            sum_dpos += psize[j];
-            min_ap = min(min_ap, ap_pool[j]);
-            sum_inv += 1.0 / max(ap_pool[j], 1);
-            if (ap && ap_pool[j] == 1) ++sole;
-            if (ap_pool[j] == 0) ++unexplained;
+    for (int e = 0; e < d; ++e) {
+        const long long j = c.base + c.row[e];
+        const int size = in.psize[j];
+        sum_d += size;
+        if (in.y[j]) {
+            const int a = in.ap_pool[j];
+            sum_dpos += size;
+            min_ap = min(min_ap, a);
+            sum_inv += 1.0 / max(a, 1);
+            if (ap && a == 1) ++sole;
+            if (a == 0) ++unexplained;
         }
     }
-    float *f = Fout + i * 16;
-    f[0] = d / 8.0f;
-    f[1] = p / 8.0f;
-    f[2] = nn / 8.0f;
-    f[3] = static_cast<float>(p) / static_cast<float>(max(d, 1));
-    f[4] = static_cast<float>((lam + p * a_pos + nn * a_neg) / 10.0);
-    f[5] = d ? static_cast<float>(sum_d / d / dbar) : 0.f;
-    f[6] = p ? static_cast<float>(sum_dpos / p / dbar) : 0.f;
-    f[7] = static_cast<float>(ap);
-    f[8] = p ? min_ap / 10.0f : 0.f;
-    f[9] = p ? static_cast<float>(sum_inv / p) : 0.f;
-    f[10] = sole / 8.0f;
-    f[11] = unexplained / 8.0f;
-    f[12] = nap[s] / 100.0f;
-    f[13] = static_cast<float>(lam / 10.0);
-    f[14] = static_cast<float>(a_pos / 10.0);
-    f[15] = static_cast<float>(a_neg / 10.0);
+    const float4 f[4] = {
+        make_float4(d / 8.0f, p / 8.0f, nn / 8.0f, static_cast<float>(p) / static_cast<float>(max(d, 1))),
+        make_float4(static_cast<float>((lam + p * a_pos + nn * a_neg) / 10.0), d ? static_cast<float>(sum_d / d / dbar) : 0.f,
+                    p ? static_cast<float>(sum_dpos / p / dbar) : 0.f, static_cast<float>(ap)),
+        make_float4(p ? min_ap / 10.0f : 0.f, p ? static_cast<float>(sum_inv / p) : 0.f, sole / 8.0f, unexplained / 8.0f),
+        make_float4(in.nap[c.s] / 100.0f, static_cast<float>(lam / 10.0), static_cast<float>(a_pos / 10.0),
+                    static_cast<float>(a_neg / 10.0))};
+    float *out = Fout + i * 16;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        if ((reinterpret_cast<uintptr_t>(Fout) & 15u) == 0) {
+            reinterpret_cast<float4 *>(out)[k] = f[k];
+        } else {                       // the caller's array need only hold floats
+            out[4 * k] = f[k].x; out[4 * k + 1] = f[k].y; out[4 * k + 2] = f[k].z; out[4 * k + 3] = f[k].w;
+        }
+    }
 }
 
 int grid_for(long long n, int block) {
@@ -438,12 +449,10 @@ int mcpd_features_batch(mcpd_ctx *ctx, int32_t n_inst, const mcpd_design *design
                         const uint8_t *const *ys, const double *rates, float *feat_dev) {
     using namespace mcpd;
     if (!ctx || n_inst < 1 || !designs || !ys || !rates || !feat_dev) return MCPD_EINVAL;
-    // Concatenate the designs: clone rows keep their local pool ids plus a per-clone pool base.
-    std::vector<int32_t> ptr(1, 0), pools, cinst;
-    std::vector<int64_t> pbase;
-    std::vector<uint8_t> y;
+    // Sizes and checks.
+    std::vector<long long> off(3 * (static_cast<size_t>(n_inst) + 1), 0);
+    long long *const clone_off = off.data(), *const entry_off = clone_off + n_inst + 1, *const pool_off = entry_off + n_inst + 1;
     std::vector<double> consts(4 * static_cast<size_t>(n_inst));
-    long long pool_off = 0;
     for (int32_t s = 0; s < n_inst; ++s) {
         const mcpd_design &d = designs[s];
         if (d.n_clones < 1 || d.n_pools < 1 || !d.clone_ptr) return fail_m(ctx, MCPD_EINVAL, "bad design");
@@ -453,59 +462,92 @@ int mcpd_features_batch(mcpd_ctx *ctx, int32_t n_inst, const mcpd_design *design
         consts[4 * s + 1] = std::log(1.0 - fn) - std::log(fp);
         consts[4 * s + 2] = std::log(fn) - std::log(1.0 - fp);
         consts[4 * s + 3] = static_cast<double>(d.clone_ptr[d.n_clones]) / d.n_pools;
-        for (int32_t i = 0; i < d.n_clones; ++i) {
-            for (int32_t e = d.clone_ptr[i]; e < d.clone_ptr[i + 1]; ++e) {
-                if (d.clone_pools[e] < 0 || d.clone_pools[e] >= d.n_pools) return fail_m(ctx, MCPD_EINVAL, "pool id");
-                pools.push_back(d.clone_pools[e]);
-            }
-            ptr.push_back(static_cast<int32_t>(pools.size()));
-            pbase.push_back(pool_off);
-            cinst.push_back(s);
-        }
-        for (int32_t j = 0; j < d.n_pools; ++j) y.push_back(ys[s][j] ? 1 : 0);
-        pool_off += d.n_pools;
+        long long entries = 0;
+        for (int32_t i = 0; i < d.n_clones; ++i) entries += std::max(0, d.clone_ptr[i + 1] - d.clone_ptr[i]);
+        clone_off[s + 1] = clone_off[s] + d.n_clones;
+        entry_off[s + 1] = entry_off[s] + entries;
+        pool_off[s + 1] = pool_off[s] + d.n_pools;
     }
-    const long long n = static_cast<long long>(cinst.size());
+    const long long n = clone_off[n_inst], entries = entry_off[n_inst], pools = pool_off[n_inst];
+    // One upload: offsets, constants, clone_ptr and clone_pools as they are, outcomes; then the device's
+    // counts.  (Pool bases and instances written per clone on the host, six pageable copies and an
+    // allocation per call took 1.5 ms for 64 instances of 1298 clones.)
+    size_t bytes = 0;
+    auto take = [&](size_t b) { const size_t at = bytes; bytes += (b + 15) / 16 * 16; return at; };
+    const size_t o_off = take(off.size() * 8), o_consts = take(consts.size() * 8), o_ptr = take((n + n_inst) * 4);
+    const size_t o_pools = take(entries * 4), o_y = take(pools), uploaded = bytes;
+    const size_t o_count = take((2 * pools + n_inst) * 4);
     CUM(cudaSetDevice(ctx->device));
-    cudaStream_t st = ctx->stream;
-    void *buf = nullptr;
-    const size_t nb = ptr.size() * 4 + pools.size() * 4 + y.size() + pbase.size() * 8 + cinst.size() * 4 +
-                      consts.size() * 8 + 4 * n * 4 + 2 * pool_off * 4 + n_inst * 4 + 1024;
-    CUM(cudaMalloc(&buf, nb));
-    char *p = static_cast<char *>(buf);
-    auto take = [&](size_t bytes) { char *at = p; p += (bytes + 15) / 16 * 16; return at; };
-    int32_t *d_ptr = reinterpret_cast<int32_t *>(take(ptr.size() * 4));
-    int32_t *d_pools = reinterpret_cast<int32_t *>(take(pools.size() * 4 + 4));
-    uint8_t *d_y = reinterpret_cast<uint8_t *>(take(y.size()));
-    int64_t *d_pbase = reinterpret_cast<int64_t *>(take(pbase.size() * 8));
-    int32_t *d_cinst = reinterpret_cast<int32_t *>(take(cinst.size() * 4));
-    double *d_consts = reinterpret_cast<double *>(take(consts.size() * 8));
-    int32_t *d_deg = reinterpret_cast<int32_t *>(take(n * 4));
-    int32_t *d_npos = reinterpret_cast<int32_t *>(take(n * 4));
-    int32_t *d_allpos = reinterpret_cast<int32_t *>(take(n * 4));
-    int32_t *d_psize = reinterpret_cast<int32_t *>(take(pool_off * 4));
-    int32_t *d_ap = reinterpret_cast<int32_t *>(take(pool_off * 4));
-    int32_t *d_nap = reinterpret_cast<int32_t *>(take(n_inst * 4));
+    if (bytes > ctx->stage_bytes) {
+        if (ctx->stage_bytes) { cudaFreeHost(ctx->stage_host); cudaFree(ctx->stage_dev); ctx->stage_bytes = 0; }
+        CUM(cudaMallocHost(&ctx->stage_host, bytes));
+        const cudaError_t e = cudaMalloc(&ctx->stage_dev, bytes);
+        if (e != cudaSuccess) { cudaFreeHost(ctx->stage_host); return fail_m(ctx, MCPD_ECUDA, "cudaMalloc"); }
+        ctx->stage_bytes = bytes;
+    }
+    char *const h = static_cast<char *>(ctx->stage_host), *const dv = static_cast<char *>(ctx->stage_dev);
+    std::memcpy(h + o_off, off.data(), off.size() * 8);
+    std::memcpy(h + o_consts, consts.data(), consts.size() * 8);
     int rc = MCPD_OK;
-    do {
-        if (cudaMemcpyAsync(d_ptr, ptr.data(), ptr.size() * 4, cudaMemcpyHostToDevice, st) != cudaSuccess ||
-            (!pools.empty() && cudaMemcpyAsync(d_pools, pools.data(), pools.size() * 4, cudaMemcpyHostToDevice, st) != cudaSuccess) ||
-            cudaMemcpyAsync(d_y, y.data(), y.size(), cudaMemcpyHostToDevice, st) != cudaSuccess ||
-            cudaMemcpyAsync(d_pbase, pbase.data(), pbase.size() * 8, cudaMemcpyHostToDevice, st) != cudaSuccess ||
-            cudaMemcpyAsync(d_cinst, cinst.data(), cinst.size() * 4, cudaMemcpyHostToDevice, st) != cudaSuccess ||
-            cudaMemcpyAsync(d_consts, consts.data(), consts.size() * 8, cudaMemcpyHostToDevice, st) != cudaSuccess ||
-            cudaMemsetAsync(d_psize, 0, pool_off * 4, st) != cudaSuccess ||
-            cudaMemsetAsync(d_ap, 0, pool_off * 4, st) != cudaSuccess ||
-            cudaMemsetAsync(d_nap, 0, n_inst * 4, st) != cudaSuccess) { rc = MCPD_ECUDA; break; }
+    for (int32_t s = 0; s < n_inst && rc == MCPD_OK; ++s) {
+        const mcpd_design &d = designs[s];
+        int32_t *ptr = reinterpret_cast<int32_t *>(h + o_ptr) + clone_off[s] + s;
+        int32_t *pl = reinterpret_cast<int32_t *>(h + o_pools) + entry_off[s];
+        uint32_t worst = 0;
+        if (entry_off[s + 1] - entry_off[s] == d.clone_ptr[d.n_clones] - d.clone_ptr[0]) {      // ascending
+            std::memcpy(ptr, d.clone_ptr, (static_cast<size_t>(d.n_clones) + 1) * 4);
+            const int32_t *src = d.clone_pools + d.clone_ptr[0];
+            for (long long e = 0, m = entry_off[s + 1] - entry_off[s]; e < m; ++e) {
+                worst = std::max(worst, static_cast<uint32_t>(src[e]));
+                pl[e] = src[e];
+            }
+        } else {                       // a falling clone_ptr: the clone has no pools
+            int32_t at = 0;
+            for (int32_t i = 0; i < d.n_clones; ++i) {
+                ptr[i] = at;
+                for (int32_t e = d.clone_ptr[i]; e < d.clone_ptr[i + 1]; ++e) {
+                    worst = std::max(worst, static_cast<uint32_t>(d.clone_pools[e]));
+                    pl[at++] = d.clone_pools[e];
+                }
+            }
+            ptr[d.n_clones] = at;
+        }
+        if (entry_off[s + 1] > entry_off[s] && worst >= static_cast<uint32_t>(d.n_pools)) rc = fail_m(ctx, MCPD_EINVAL, "pool id");
+        std::memcpy(h + o_y + pool_off[s], ys[s], static_cast<size_t>(d.n_pools));
+    }
+    if (rc == MCPD_OK) {
+        cudaStream_t st = ctx->stream;
+        FeatIn in;
+        in.clone_off = reinterpret_cast<const long long *>(dv + o_off);
+        in.entry_off = in.clone_off + n_inst + 1;
+        in.pool_off = in.entry_off + n_inst + 1;
+        in.consts = reinterpret_cast<const double *>(dv + o_consts);
+        in.ptr = reinterpret_cast<const int32_t *>(dv + o_ptr);
+        in.pools = reinterpret_cast<const int32_t *>(dv + o_pools);
+        in.y = reinterpret_cast<const uint8_t *>(dv + o_y);
+        in.n_inst = n_inst;
+        in.psize = reinterpret_cast<int32_t *>(dv + o_count);
+        in.ap_pool = in.psize + pools;
+        in.nap = in.ap_pool + pools;
         const int g = grid_for(n, 256);
-        feat_pass1<<<g, 256, 0, st>>>(n, d_ptr, d_pools, d_y, d_pbase, d_deg, d_npos, d_allpos, d_psize, d_nap, d_cinst);
-        feat_pass2<<<g, 256, 0, st>>>(n, d_ptr, d_pools, d_pbase, d_allpos, d_ap);
-        feat_pass3<<<g, 256, 0, st>>>(n, d_ptr, d_pools, d_y, d_pbase, d_deg, d_npos, d_allpos, d_psize, d_ap,
-                                      d_nap, d_cinst, d_consts, feat_dev);
-        if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess) rc = MCPD_ECUDA;
-    } while (0);
-    cudaFree(buf);
-    return rc == MCPD_OK ? MCPD_OK : fail_m(ctx, rc, "features kernels");
+        if (cudaMemcpyAsync(dv, h, uploaded, cudaMemcpyHostToDevice, st) != cudaSuccess ||
+            cudaMemsetAsync(in.psize, 0, (2 * pools + n_inst) * 4, st) != cudaSuccess) {
+            rc = MCPD_ECUDA;
+        } else {
+            feat_counts<<<g, 256, 0, st>>>(n, in);
+            feat_rows<<<g, 256, 0, st>>>(n, in, feat_dev);
+            if (cudaGetLastError() != cudaSuccess) rc = MCPD_ECUDA;
+        }
+        if (cudaStreamSynchronize(st) != cudaSuccess) rc = MCPD_ECUDA;
+        if (rc != MCPD_OK) fail_m(ctx, rc, "features kernels");
+    }
+    if (ctx->stage_bytes > kKeepStaging) {
+        cudaFreeHost(ctx->stage_host);
+        cudaFree(ctx->stage_dev);
+        ctx->stage_host = ctx->stage_dev = nullptr;
+        ctx->stage_bytes = 0;
+    }
+    return rc;
 }
 
 int mcpd_mlp_forward(mcpd_ctx *ctx, int64_t n_rows, const float *X, const uint16_t *W, float *Out) {

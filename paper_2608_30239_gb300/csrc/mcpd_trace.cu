@@ -44,23 +44,12 @@ TraceFn pick_trace(int coupled, int scan, int udeg) {
 
 }  // namespace
 
-int set_trace_smem(size_t bytes) {
-    for (int c = 0; c <= 1; ++c)
-        for (int sc : {MCPD_SCAN_SCORE, MCPD_SCAN_SYSTEMATIC}) {
-            if (c && sc == MCPD_SCAN_SYSTEMATIC) continue;
-            for (int ud = 0; ud <= 8; ++ud) {
-                if (ud == 1 || ud == 2 || (!c && ud > kMaskDeg)) continue;
-                if (cudaFuncSetAttribute(pick_trace(c, sc, ud), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(bytes)) != cudaSuccess)
-                    return MCPD_ECUDA;
-            }
-        }
-    return MCPD_OK;
-}
-
 int launch_pairs_trace(const KParams &kp, int grid, int block, size_t smem, void *stream) {
     if (!kp.trace_rec || kp.trace_stride <= 0) return MCPD_EINVAL;
     const BParams none{};
+    if (cudaFuncSetAttribute(pick_trace(kp.coupled, kp.scan, kp.udeg), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             static_cast<int>(smem)) != cudaSuccess)
+        return MCPD_ECUDA;
     pick_trace(kp.coupled, kp.scan, kp.udeg)<<<grid, block, smem, static_cast<cudaStream_t>(stream)>>>(kp, none);
     return cudaGetLastError() == cudaSuccess ? MCPD_OK : MCPD_ECUDA;
 }

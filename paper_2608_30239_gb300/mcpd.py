@@ -128,7 +128,7 @@ def _ptr(a):
         return None
     if hasattr(a, "data_ptr"):
         return C.c_void_p(a.data_ptr())
-    return a.ctypes.data_as(C.c_void_p)
+    return C.c_void_p(a.ctypes.data)
 
 
 def _check_out(est, se, need, device):
