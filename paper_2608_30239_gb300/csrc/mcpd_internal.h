@@ -59,10 +59,10 @@ enum PairStat {
 #endif
 MCPD_HD inline long long pair_words(long long na, long long W) { return 2 * na + kPairStats + W; }
 // Sampling kernel: an entry is one slot's sums G [na]; a warp's scratch is `bank` entries, the list
-// of those whose pairs are done (three 32-bit words each), a statistics record per lane and, coupled,
+// of those whose pairs are done (two 32-bit words each), a statistics record per lane and, coupled,
 // sums per pair (at most 16, and one per slot of a chunk).  In 8-byte words.
 MCPD_HD inline long long warp_words(long long bank, long long na, bool coupled) {
-    return bank * na + (3 * bank + 1) / 2 + 32 * kPairStats + (coupled ? (bank < 16 ? bank : 16) * na : 0);
+    return bank * na + bank + 32 * kPairStats + (coupled ? (bank < 16 ? bank : 16) * na : 0);
 }
 #undef MCPD_HD
 

@@ -79,10 +79,10 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
     const size_t ew = static_cast<size_t>(stride_na);
     auto list = [&]() { return reinterpret_cast<uint32_t *>(wbase + bank * ew); };
     auto pst = [&]() {
-        return reinterpret_cast<unsigned long long *>(wbase + bank * ew + (3 * bank + 1) / 2 + lane * kPairStats);
+        return reinterpret_cast<unsigned long long *>(wbase + bank * ew + bank + lane * kPairStats);
     };
     // Pair i's events of the replication it is running.
-    auto pair_sums = [&](int i) { return wbase + bank * ew + (3 * bank + 1) / 2 + 32 * kPairStats + i * ew; };
+    auto pair_sums = [&](int i) { return wbase + bank * ew + bank + 32 * kPairStats + i * ew; };
     unsigned long long *const counters = BATCH ? bp.counters : p.counters;
 #pragma unroll
     for (int i = 0; i < kPairStats; ++i) pst()[i] = 0ull;
@@ -171,7 +171,7 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
     bool on = false;                      // takes steps
     bool dirty = false;                   // some bit of its column may be set
     bool events = false;                  // its pair's sums may hold something
-    uint32_t slot_local = 0, slot_g = 0, r = 0, t = 0, S = 0, N = 0, D = 0, stop = 0, item = 0;
+    uint32_t slot_local = 0, slot_g = 0, r = 0, t = 0, S = 0, N = 0, D = 0, stop = 0;
     long long *sum = nullptr;             // where its events go: the slot's entry, or its pair's sums
     int32_t *trec = nullptr;              // TRACE: the record of the current replication
     uint32_t trace_from = 0;              // TRACE: the single run records from its pair's meeting on
@@ -242,12 +242,14 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
         for (int l = 0; l < kRow; ++l)
             if (real(l, s.ent)) cbase[s.ent[l]] = static_cast<unsigned char>(s.c[l] + delta);
     };
+    uint32_t first = 0, cnt = 0;          // the chunk: slots first .. first + cnt - 1
+
     // Random start Z_0 ~ prod Bernoulli(nu_i) of lane src's new replication, drawn by the whole
     // warp: the lanes take the clone pairs that have some nu_i > 0 (one Philox block each, tag 1, counter
-    // (a / 2, r, slot, instance)) and set the bits and pool counts they draw in src's column with
-    // shared-memory atomics (a count word holds four pools of one column, and a count never
-    // passes 255, so adding 1 << 8 b touches only its own byte).
-    auto coop_init = [&](int src) {
+    // (a / 2, r, slot, instance)) and set the bits and pool counts they draw in src's column, and for
+    // a pair (X_0 = Y_0) in Y's, with shared-memory atomics (a count word holds four pools of one
+    // column, and a count never passes 255, so adding 1 << 8 b touches only its own byte).
+    auto coop_init = [&](int src, bool both) {
         const uint32_t r_s = __shfl_sync(FULL, r, src), slot_s = __shfl_sync(FULL, slot_g, src);
         uint32_t *const st_s = st - lane + src;
         unsigned char *const cb_s = reinterpret_cast<unsigned char *>(st_s);
@@ -265,89 +267,84 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
                                                : ((static_cast<unsigned long long>(b.x) << 32) | b.y);
                 if (u < __ldg(tnu + c)) {
                     atomicOr(&st_s[(c >> 5) * 32], 1u << (c & 31));
+                    if (both) atomicOr(&st_s[(c >> 5) * 32 + 16], 1u << (c & 31));
                     uint32_t ent[8];
                     entries(rowAt(c), ent);
 #pragma unroll
                     for (int l = 0; l < kRow; ++l) {
                         if (!real(l, ent)) continue;
-                        const uint32_t off = ent[l];
-                        atomicAdd(reinterpret_cast<uint32_t *>(cb_s + (off & ~3u)), 1u << (8u * (off & 3u)));
+                        const uint32_t off = ent[l], one = 1u << (8u * (off & 3u));
+                        uint32_t *const word = reinterpret_cast<uint32_t *>(cb_s + (off & ~3u));
+                        atomicAdd(word, one);
+                        if (both) atomicAdd(word + 16, one);
                     }
                 }
             }
         }
         __syncwarp();
     };
-    // Start the replications of the lanes in `who` (their columns are empty).
+    // Random starts of the new replications of the lanes with `mine` (their columns are empty).
     auto start_random = [&](bool mine) {
         if (v_Tnu() == nullptr) return;
-        unsigned m = __ballot_sync(FULL, mine);
+        const unsigned all = __ballot_sync(FULL, mine), pair = __ballot_sync(FULL, mine && role >= 2);
+        unsigned m = all & ~(pair & 0xFFFF0000u);
         __syncwarp();
         while (m) {
             const int src = __ffs(m) - 1;
             m &= m - 1;
-            coop_init(src);
+            coop_init(src, (pair >> src) & 1u);
         }
         if (mine) dirty = true;
     };
-    // Empty lane src's column by the whole warp; `w` != 0: first add w for every bit set (the closing
-    // term of a single run) to its entry.
-    auto coop_clear = [&](int src, uint32_t w) {
+    // Empty lane src's column, and for a pair (`both`) Y's, by the whole warp; `w` != 0: first add w
+    // for every bit set (the closing term of a single run) to its entry.
+    auto coop_clear = [&](int src, bool both, uint32_t w) {
         const uint32_t w_s = __shfl_sync(FULL, w, src);
         long long *const sum_s = reinterpret_cast<long long *>(__shfl_sync(FULL, reinterpret_cast<unsigned long long>(sum), src));
         uint32_t *const st_s = st - lane + src;
         for (uint32_t q = lane, e = v_wpp(); q < e; q += 32) {
             if (q < W && w_s) {
-                const uint32_t xw = st_s[q * 32];
-                uint32_t m = xw;
+                uint32_t m = st_s[q * 32];
                 while (m) {
                     const int b = __ffs(m) - 1;
                     m &= m - 1;
                     red_add(sum_s + q * 32 + b, static_cast<long long>(w_s));
                 }
             }
-            st_s[q * 32] = (DEG == 0 && q == v_dwi()) ? v_dw() : 0u;
+            const uint32_t v = (DEG == 0 && q == v_dwi()) ? v_dw() : 0u;
+            st_s[q * 32] = v;
+            if (both) st_s[q * 32 + 16] = v;
         }
         __syncwarp();
     };
-    // Add the entries of the lanes with `mine` to bucket N - 1 (N = 0: the slot is dropped) and zero
-    // them, each by the whole warp: coalesced reads of all its sums, four in flight a lane.  (Marking
-    // the touched clones with a reduction per flip, to read only those here, cost every flip more
-    // than reading na sums once per slot.)  The reductions of every lane into these entries are
-    // performed before they are read, and the zeros before a later slot reduces into them.
-    auto flush = [&](bool mine, uint32_t n) {
-        __threadfence();
-        unsigned m = __ballot_sync(FULL, mine);
-        __syncwarp();
-        while (m) {
-            const int src = __ffs(m) - 1;
-            m &= m - 1;
-            const uint32_t n_s = __shfl_sync(FULL, n, src), slot_s = __shfl_sync(FULL, slot_local, src);
-            long long *const sum_s = reinterpret_cast<long long *>(__shfl_sync(FULL, reinterpret_cast<unsigned long long>(sum), src));
-            long long *tr = nullptr;
-            if constexpr (!BATCH) {
-                if (n_s && p.trace_stride > 0 && (slot_s % p.trace_stride) == 0)
-                    tr = p.trace_G + (static_cast<long long>(slot_s) / p.trace_stride) * na;
-            }
-            for (int j0 = lane; j0 < na; j0 += 128) {
-                long long g[4];
+    // Add entry `idx` to bucket n - 1 (n = 0: the slot is dropped) and zero it, by the whole warp:
+    // coalesced reads of all its sums, four in flight a lane.  (Marking the touched clones with a
+    // reduction per flip, to read only those here, cost every flip more than reading na sums once
+    // per slot.)
+    auto flush = [&](uint32_t idx, uint32_t n) {
+        long long *const from = wbase + static_cast<size_t>(idx) * ew;
+        const uint32_t slot = first + idx;
+        long long *tr = nullptr;
+        if constexpr (!BATCH) {
+            if (n && p.trace_stride > 0 && (slot % p.trace_stride) == 0)
+                tr = p.trace_G + (static_cast<long long>(slot) / p.trace_stride) * na;
+        }
+        for (int j0 = lane; j0 < na; j0 += 128) {
+            long long g[4];
 #pragma unroll
-                for (int u = 0; u < 4; ++u) g[u] = j0 + 32 * u < na ? __ldcg(sum_s + j0 + 32 * u) : 0;
+            for (int u = 0; u < 4; ++u) g[u] = j0 + 32 * u < na ? __ldcg(from + j0 + 32 * u) : 0;
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    if (g[u] == 0) continue;
-                    const int j = j0 + 32 * u;
-                    sum_s[j] = 0;
-                    if (n_s) {
-                        bucket_add(v_S1(), v_S2lo(), v_S2hi(), na, static_cast<int>(n_s) - 1, j, g[u]);
-                        if (tr) tr[j] = g[u];
-                    }
+            for (int u = 0; u < 4; ++u) {
+                if (g[u] == 0) continue;
+                const int j = j0 + 32 * u;
+                from[j] = 0;
+                if (n) {
+                    bucket_add(v_S1(), v_S2lo(), v_S2hi(), na, static_cast<int>(n) - 1, j, g[u]);
+                    if (tr) tr[j] = g[u];
                 }
             }
-            if (lane == src && n_s) atomicAdd(&v_bcount()[n_s - 1], 1ull);
         }
-        __threadfence();
-        __syncwarp();
+        if (lane == 0 && n) atomicAdd(&v_bcount()[n - 1], 1ull);
     };
     auto record_slot = [&](uint32_t nstar, long long cost, uint32_t reps) {
         if constexpr (!BATCH) {
@@ -380,7 +377,6 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
         }
     };
     // Point the lane at slot `idx` of the chunk and its entry.
-    uint32_t first = 0, cnt = 0;          // the chunk: slots first .. first + cnt - 1
     auto entry = [&]() { return wbase + static_cast<size_t>(slot_local - first) * ew; };
     auto take = [&](uint32_t idx) {
         slot_local = first + idx;
@@ -428,32 +424,34 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
         }
         // Single runs, the chunk's (slot, replication) pairs: any lane takes any of them, for a
         // slot's sums take reductions from every lane.  The list holds, per slot whose pairs are done,
-        // its entry, N and how many of its N runs are left (the last one flushes the entry); head and
-        // hr are the next run's.
-        uint32_t head = 0, hr = 0, ready = 0;
+        // its entry and N (0: dropped); run_n, run_idx are the head's (read once per slot), hr its next
+        // replication.
+        uint32_t head = 0, hr = 0, ready = 0, run_n = 0, run_idx = 0;
         role = 0; on = false;
         auto assign_runs = [&]() -> bool {
             bool got = false;
-            while (head < ready) {
+            for (;;) {
                 const unsigned idle = __ballot_sync(FULL, role == 0);
                 if (!idle) break;
-                const uint32_t n = __ldcg(list() + 3 * head + 1);
-                const uint32_t k = min(n - hr, static_cast<uint32_t>(__popc(idle)));
+                if (hr == run_n) {
+                    if (head == ready) break;
+                    run_idx = __ldcg(list() + 2 * head);
+                    run_n = __ldcg(list() + 2 * head + 1);
+                    hr = 0;
+                    ++head;
+                }
+                const uint32_t k = min(run_n - hr, static_cast<uint32_t>(__popc(idle)));
                 const uint32_t rank = __popc(idle & ((1u << lane) - 1u));
                 if (role == 0 && rank < k) {
-                    take(__ldcg(list() + 3 * head));
-                    N = n;
+                    take(run_idx);
                     r = hr + rank;
-                    item = head;
                     role = 1;
                     got = true;
                 }
                 hr += k;
-                if (hr == n) { ++head; hr = 0; }
             }
             return got;
         };
-        auto last_run = [&]() -> bool { return atomicSub(list() + 3 * item + 2, 1u) == 1u; };
 
         // ---- Phase 1: pairs to their meetings, and single runs on the lanes that are left over.
         if constexpr (COUPLED) {
@@ -522,13 +520,12 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
                 if (begin || __any_sync(FULL, ended)) {
                     begin = false;
                     __syncwarp();         // the columns as every lane's steps left them
-                    bool restart = false, out = false, done = false, banked = false, keep = false;
+                    bool restart = false, done = false, banked = false, keep = false;
                     uint32_t close = 0;
                     const bool pair_ended = ended && role >= 2;
                     if (ended) {
                         if (role == 1) {
                             close = wstep(ell);
-                            out = last_run();
                             done = true;
                         } else {
                             // 1 completed (met, or unmet at the meeting cap), 2 doomed (it cannot end
@@ -572,7 +569,6 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
                                 if (S < B && B - S >= v_unit()) { ++r; restart = true; } else over = true;
                             } else {
                                 over = true;
-                                out = how == 3 && role == 2;      // the slot is dropped
                             }
                             if (over) {
                                 if (role == 2) {
@@ -588,8 +584,9 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
                                         stat_add(kPsLimit, 1);
                                         atomicExch(BATCH ? bp.error : p.error, 1);
                                     }
-                                    record_slot(how == 3 ? 0u : N, static_cast<long long>(S), r + 1);
-                                    banked = how != 3;
+                                    if (how == 3) N = 0;          // the slot is dropped
+                                    record_slot(N, static_cast<long long>(S), r + 1);
+                                    banked = true;
                                 }
                                 done = true;
                             }
@@ -626,34 +623,29 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
                             __syncwarp();
                             if (pair_ended) events = false;
                         }
-                        if (pair_ended && done) sum = entry();
                     }
-                    // columns of the ended lanes (a lane that never flipped has an empty one)
+                    // columns of the ended lanes (where nothing flipped they are empty)
                     {
-                        const bool mine = (restart || done) && dirty;
-                        unsigned m = __ballot_sync(FULL, mine);
+                        const unsigned pair = __ballot_sync(FULL, pair_ended && dirty);
+                        unsigned m = __ballot_sync(FULL, ended && role == 1 && dirty) | ((pair | pair >> 16) & 0xFFFFu);
                         __syncwarp();
                         while (m) {
                             const int src = __ffs(m) - 1;
                             m &= m - 1;
-                            coop_clear(src, close);
+                            coop_clear(src, ((pair | pair >> 16) >> src) & 1u, close);
                         }
-                        if (mine) dirty = false;
+                        if (ended) dirty = false;
                     }
-                    // entries: a slot whose pairs are done goes on the list, one that is over to its bucket
+                    // a slot whose pairs are done goes on the list
                     {
                         const unsigned m = __ballot_sync(FULL, banked);
-                        if (m) {
-                            if (banked) {
-                                const uint32_t at = ready + __popc(m & ((1u << lane) - 1u));
-                                list()[3 * at] = slot_local - first;
-                                list()[3 * at + 1] = N;
-                                list()[3 * at + 2] = N;
-                            }
-                            ready += __popc(m);
-                            __syncwarp();
+                        if (banked) {
+                            const uint32_t at = ready + __popc(m & ((1u << lane) - 1u));
+                            list()[2 * at] = slot_local - first;
+                            list()[2 * at + 1] = N;
                         }
-                        if (__any_sync(FULL, out)) flush(out, role == 1 ? N : 0u);
+                        ready += __popc(m);
+                        __syncwarp();
                         if (done) role = 0;
                     }
                     // free lanes: pairs for the slots that are left, then single runs
@@ -707,9 +699,8 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
             const uint32_t B = v_B(), n = max(1u, B / ell);      // ell: a chain's b + T - 1 >= 1 steps
             for (uint32_t idx = lane; idx < cnt; idx += 32) {
                 take(idx);
-                list()[3 * idx] = idx;
-                list()[3 * idx + 1] = n;
-                list()[3 * idx + 2] = n;
+                list()[2 * idx] = idx;
+                list()[2 * idx + 1] = n;
                 stat_add(kPsProgress, static_cast<unsigned long long>(n) * ell);
                 stat_add(kPsSiteUpdates, static_cast<unsigned long long>(n) * ell);
                 stat_add(kPsStarted, n);
@@ -818,10 +809,16 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
                 }
             }
             __syncwarp();
-            const bool out = role == 1 && last_run();
-            if (__any_sync(FULL, out)) flush(out, N);
             role = 0;
         }
+
+        // ---- The chunk's sums to their buckets: every lane's reductions into the entries are performed
+        // before they are read, and the zeros before the next chunk reduces into them.
+        __threadfence();
+        __syncwarp();
+        for (uint32_t at = 0; at < ready; ++at) flush(__ldcg(list() + 2 * at), __ldcg(list() + 2 * at + 1));
+        __threadfence();
+        __syncwarp();
     }
 
     // Every lane of the warp is here: sum (or max) the lanes' statistics over the warp.
