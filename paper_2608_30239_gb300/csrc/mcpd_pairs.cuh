@@ -385,12 +385,16 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
         r = 0;
     };
 
-    for (;;) {
-        // The next chunk of slots (one atomic per chunk).
+    for (bool begin = true;; begin = false) {
+        // The next chunk of slots.  The first one is the warp's own number, so that a block's warps
+        // start on neighbouring chunks (in a batch mostly one instance, whose tables they share
+        // through the L1); the rest from one counter.
         {
-            unsigned long long s = 0;
-            if (lane == 0) s = atomicAdd(&counters[kWork], 1ull);
-            s = __shfl_sync(FULL, s, 0);
+            unsigned long long s = blockIdx.x * static_cast<unsigned>(nwarps) + static_cast<unsigned>(warp);
+            if (!begin) {
+                if (lane == 0) s = atomicAdd(&counters[kWork], 1ull);
+                s = __shfl_sync(FULL, s, 0) + static_cast<unsigned long long>(gridDim.x) * static_cast<unsigned>(nwarps);
+            }
             if constexpr (!BATCH) {
                 const unsigned long long at = s * static_cast<unsigned long long>(p.chunk);
                 if (at >= static_cast<unsigned long long>(p.P)) break;
