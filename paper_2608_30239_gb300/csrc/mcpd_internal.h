@@ -66,8 +66,12 @@ MCPD_HD inline long long warp_words(long long bank, long long na, bool coupled) 
 }
 #undef MCPD_HD
 
-// Threads per block the sampling kernel is compiled for.
-constexpr int pairs_threads(int deg, bool batch) { return batch || deg == 0 || deg > kMaskDeg ? 640 : 768; }
+// Threads per block the sampling kernel is compiled for: 20 warps of 96 registers, and 16 of 128 for the
+// builds with eight row entries or a batch's descriptors.  More warps lose more to the registers they
+// take than they hide: 24 warps of 80 registers against 20 of 96, 1298 x 97 at high noise, 105.5 against
+// 94.7 ms (low noise 24.9 and 22.3, a learned start 21.0 and 18.3); 18 of 112: 103.4 ms; 16 of 128:
+// 108.4.  Batches at 20 of 96 against 16 of 128: 128 uneven instances 67.0 against 60.8 ms.
+constexpr int pairs_threads(int deg, bool batch) { return batch || deg == 0 || deg > kMaskDeg ? 512 : 640; }
 
 // Everything the sampler needs, built on the host from (design, y, params).
 struct Tables {
