@@ -2,6 +2,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstdio>
 #include <cstring>
 #include <new>
@@ -699,11 +700,14 @@ int batch_shape(mcpd_ctx *ctx, mcpd_batch *b, int warps, int lanes = 1) {
             w = shape.warps;
             c.smem = shape.smem;
             per_sm = shape.per_sm;
-            // The class's part of the GPU's warps, and the slots that makes for each.
+            // The class's part of the GPU's warps, and the slots that makes for each: its chunk, up to 64.
+            // Beyond that chunks of 32, so that the short slots' warps take more of them than the
+            // long ones' (128 uneven instances, whole shares against 32: 512 slots 58.8 against 60.8 ms,
+            // 1024 slots 109.7 against 91.6 ms).
             const long long resident = static_cast<long long>(ctx->sm_count) * per_sm * w;
             const double part = work > 0 ? static_cast<double>(class_slots) * c.bp.max_wpp / work : 1.0;
-            c.bp.bank = static_cast<int32_t>(std::max<long long>(1, std::min<long long>(32, static_cast<long long>(
-                class_slots / std::max(1.0, resident * part)) + 1)));
+            const double share = class_slots / std::max(1.0, resident * part);
+            c.bp.bank = static_cast<int32_t>(std::max(1.0, share <= 64.0 ? std::ceil(share) : 32.0));
             long long units = 0;
             for (int32_t k = 0; k < c.count; ++k)
                 units += (b->insts0[static_cast<size_t>(c.first) + k].P + c.bp.bank - 1) / c.bp.bank;
