@@ -31,7 +31,7 @@ constexpr size_t kKeepStaging = size_t(32) << 20;
 constexpr int kRow = 8;              // pool entries per clone row (one 16-byte shared load)
 constexpr int kTSide = kRow + 1;     // acceptance table is kTSide x kTSide, indexed 9 n+ + n-
 constexpr int kMaskDeg = 6;          // uniform degrees up to this use mask-indexed thresholds
-constexpr int kBank = 160;           // slots of a chunk, at most
+constexpr int kBank = 96;            // slots of a chunk, at most
 constexpr int kMaxClones = 65535;
 constexpr int kMaxPools = 1022;      // pool byte offsets must fit 16 bits
 constexpr int kMaxPoolSize = 255;    // per-pool counts are bytes
