@@ -127,7 +127,7 @@ constexpr int BWD_SMEM = (SPARAM + H * H + (F + 4 * H) * LD + 2 * TR) * 4;
 // to dZ2 and dZ1, and gW1 = dZ1^T X, gb1 = sum dZ1, gW2 = dZ2^T H1, gb2 = sum dZ2, gW3 = dOut^T H2,
 // gb3 = sum dOut summed over the chunk's rows in registers, in row order; nothing per row goes to
 // memory.  A thread owns 16 entries of gW2 and 4 of gW1 (features 16 apart: conflict-free loads), and
-// one of gb1, gb2 or gW3.
+// one of gb1, gb2 or gW3; two warps take gb3.
 __global__ void __launch_bounds__(TB) mlp_backward_kernel(long long n, long long chunk, const float *X, const __nv_bfloat16 *W,
                                                           const float *dOut, float *partials) {
     extern __shared__ __align__(16) float sm[];
@@ -200,8 +200,7 @@ __global__ void __launch_bounds__(TB) mlp_backward_kernel(long long n, long long
                     gs = fmaf(d[r + 2], v.z, gs); gs = fmaf(d[r + 3], v.w, gs);
                 }
             }
-            if (k < O)
-                for (int r = 0; r < TR; ++r) g3 += sO[k * TR + r];
+            if (k < TR) g3 += sO[(k >> 5) * TR + (k & 31)] + sO[(k >> 5) * TR + (k & 31) + 32];   // warp o: output o
         }
     }
     float *out = partials + static_cast<long long>(blockIdx.x) * NPARAM;
@@ -213,7 +212,10 @@ __global__ void __launch_bounds__(TB) mlp_backward_kernel(long long n, long long
     }
     const int k = threadIdx.x;
     out[k < H ? OFF_B1 + k : k < 2 * H ? OFF_B2 + k - H : OFF_W3 + k - 2 * H] = gs;
-    if (k < O) out[OFF_B3 + k] = g3;
+    if (k < TR) {
+        for (int w = 16; w > 0; w >>= 1) g3 += __shfl_down_sync(0xFFFFFFFFu, g3, w);
+        if ((k & 31) == 0) out[OFF_B3 + (k >> 5)] = g3;
+    }
 }
 
 // grad[k] = the sum of the chunks' partials: 8 threads per parameter take every eighth chunk, then
