@@ -9,7 +9,7 @@ N*_p buckets are summed and theta_CT and its standard errors are finalized on th
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl reference]
 
-Prints one JSON line (rank 0).  `value` counts single-site updates executed by the sampling kernel
+Prints one JSON line (rank 0).  `value` counts the method's single-site updates
 (two per coupled draw, one for each replication's pre-lag draw) per second of device time with the
 tables resident on the GPU; `e2e` is the same metric through mcpd_decode from host arrays to host
 arrays.  The reference arm times the CPU oracle on the host's cores on a bounded slot sample.
@@ -35,9 +35,9 @@ BUDGET = 4e10
 SEED = 20260
 # DRAM bytes (read + written) per coupled draw of the sampling kernel on this workload, from one
 # ncu capture (dram__bytes_read.sum + dram__bytes_write.sum) of the 87,552-slot case of this
-# configuration (3.294e9 draws, 2.200 + 3.262 GB), scaled to a launch by its draws.  Taken for the
+# configuration (3.294e9 draws, 2.861 + 0.324 GB), scaled to a launch by its draws.  Taken for the
 # current kernel revision; it is the accumulator events and flushes, not a per-step stream.
-DRAM_BYTES_PER_DRAW = 1.6582
+DRAM_BYTES_PER_DRAW = 0.9667
 
 
 def workload_config(extra=None):

@@ -5,8 +5,8 @@ Two levels:
     candidate shapes on the batch); `tuned_shape` remembers its choice in a JSON cache keyed by GPU
     name and a coarse shape bucket (instance count, largest n_active, total slots, size classes),
     so a batch of the same shape reuses it.  Warps per block are an upper bound per size class: 0
-    lets every class take all that fit (the 20-warp kernel variant where more than 12 fit), 12
-    keeps every class on the 12-warp variant;
+    lets every class take all that fit (at most 16), 12 leaves a few idle where the fewer resident
+    slots suit the L1;
   - slots per instance at a fixed budget (`tuned_slots`): the estimator is unbiased for any number
     of slots P and horizon B (Theorem 2), so a workload that fixes each instance's budget P x B can
     take the P whose batch decodes fastest.  Each candidate is built, its shape tuned, one decode

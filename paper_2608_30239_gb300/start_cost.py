@@ -3,7 +3,7 @@
   python -m paper_2608_30239_gb300.start_cost [--slots 262144] [--reps 3]
 
 Decodes the high-noise 1298 x 97 k = 6 bench instance (horizon B = 38146, seed 7) with
-(a) nu = 0 everywhere (no draws: the build without the random-start check),
+(a) nu = 0 everywhere (no draws),
 (b) nu = 1e-4 on the 32, 164 and 656 highest-score clones (a draw per clone pair at every
     replication start, almost never a positive: the chains match (a), so the difference is the
     cost of drawing),
