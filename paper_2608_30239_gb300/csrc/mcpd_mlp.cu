@@ -56,23 +56,53 @@ __device__ __forceinline__ void stage_rows(long long n, long long r0, const floa
     }
 }
 
+// Two fp32 values in a register pair; fma2 is an fmaf of each (one instruction issues both).  The gradient's
+// products pair rows, the layers' outputs: backward 98.5 -> 94.3 us for 83,072 rows, 4.70 -> 4.28 ms for 5e6.
+using f2 = unsigned long long;
+__device__ __forceinline__ f2 pack(float x, float y) {
+    f2 v;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(x), "f"(y));
+    return v;
+}
+__device__ __forceinline__ float2 unpack(f2 v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
+    f2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+
 // acc[i][j] = bias[c0 + j] + sum_k A[k][r0 + i] B[k][c0 + j], k ascending.
 template <int K>
 __device__ __forceinline__ void tile_gemm(const float *A, const float *B, const float *bias, int r0, int c0, float (&acc)[4][4]) {
+    f2 sum[4][2];
 #pragma unroll
-    for (int j = 0; j < 4; ++j)
+    for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int i = 0; i < 4; ++i) acc[i][j] = bias ? bias[c0 + j] : 0.f;
+        for (int j = 0; j < 2; ++j) sum[i][j] = bias ? pack(bias[c0 + 2 * j], bias[c0 + 2 * j + 1]) : 0ull;
 #pragma unroll 8
     for (int k = 0; k < K; ++k) {
         const float4 a = *reinterpret_cast<const float4 *>(A + k * LD + r0);
-        const float4 b = *reinterpret_cast<const float4 *>(B + k * H + c0);
-        const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
+        const ulonglong2 b = *reinterpret_cast<const ulonglong2 *>(B + k * H + c0);
+        const float av[4] = {a.x, a.y, a.z, a.w};
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(bv[j], av[i], acc[i][j]);
+        for (int i = 0; i < 4; ++i) {
+            const f2 ai = pack(av[i], av[i]);
+            sum[i][0] = fma2(b.x, ai, sum[i][0]);
+            sum[i][1] = fma2(b.y, ai, sum[i][1]);
+        }
     }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const float2 v = unpack(sum[i][j]);
+            acc[i][2 * j] = v.x;
+            acc[i][2 * j + 1] = v.y;
+        }
 }
 // out[c0 + j][r0 + i] = f(acc[i][j])
 template <typename Fn>
@@ -137,7 +167,8 @@ __global__ void __launch_bounds__(TB) mlp_backward_kernel(long long n, long long
     for (int i = threadIdx.x; i < H * H; i += TB) sW2[i] = __bfloat162float(W[OFF_W2 + i]);   // [out][in]
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4, c0 = tx * 4, r0 = ty * 4;
     const auto relu = [](float v, int, int) { return fmaxf(v, 0.f); };
-    float g2[4][4] = {}, g1[4] = {}, gs = 0.f, g3 = 0.f;
+    f2 g2[4][4] = {}, g1[4] = {};                                 // sums of the even rows and of the odd ones
+    float gs = 0.f, g3 = 0.f;
     const long long begin = static_cast<long long>(blockIdx.x) * chunk, end = min(n, begin + chunk);
     for (long long row = begin; row < end; row += TR) {
         __syncthreads();
@@ -163,27 +194,23 @@ __global__ void __launch_bounds__(TB) mlp_backward_kernel(long long n, long long
         __syncthreads();
 #pragma unroll 2
         for (int r = 0; r < TR; r += 4) {
-            float4 d2[4], h1[4], d1[4];
+            ulonglong2 d2[4], h1[4], d1[4];
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                d2[i] = *reinterpret_cast<const float4 *>(sD2 + (ty + 16 * i) * LD + r);
-                h1[i] = *reinterpret_cast<const float4 *>(sH1 + (tx + 16 * i) * LD + r);
-                d1[i] = *reinterpret_cast<const float4 *>(sD1 + (ty + 16 * i) * LD + r);
+                d2[i] = *reinterpret_cast<const ulonglong2 *>(sD2 + (ty + 16 * i) * LD + r);
+                h1[i] = *reinterpret_cast<const ulonglong2 *>(sH1 + (tx + 16 * i) * LD + r);
+                d1[i] = *reinterpret_cast<const ulonglong2 *>(sD1 + (ty + 16 * i) * LD + r);
             }
-            const float4 x = *reinterpret_cast<const float4 *>(sX + tx * LD + r);
+            const ulonglong2 x = *reinterpret_cast<const ulonglong2 *>(sX + tx * LD + r);
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    g2[i][j] = fmaf(d2[i].x, h1[j].x, g2[i][j]);
-                    g2[i][j] = fmaf(d2[i].y, h1[j].y, g2[i][j]);
-                    g2[i][j] = fmaf(d2[i].z, h1[j].z, g2[i][j]);
-                    g2[i][j] = fmaf(d2[i].w, h1[j].w, g2[i][j]);
+                    g2[i][j] = fma2(d2[i].x, h1[j].x, g2[i][j]);
+                    g2[i][j] = fma2(d2[i].y, h1[j].y, g2[i][j]);
                 }
-                g1[i] = fmaf(d1[i].x, x.x, g1[i]);
-                g1[i] = fmaf(d1[i].y, x.y, g1[i]);
-                g1[i] = fmaf(d1[i].z, x.z, g1[i]);
-                g1[i] = fmaf(d1[i].w, x.w, g1[i]);
+                g1[i] = fma2(d1[i].x, x.x, g1[i]);
+                g1[i] = fma2(d1[i].y, x.y, g1[i]);
             }
         }
         {
@@ -207,8 +234,12 @@ __global__ void __launch_bounds__(TB) mlp_backward_kernel(long long n, long long
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
 #pragma unroll
-        for (int j = 0; j < 4; ++j) out[OFF_W2 + (ty + 16 * i) * H + tx + 16 * j] = g2[i][j];
-        out[OFF_W1 + (ty + 16 * i) * F + tx] = g1[i];
+        for (int j = 0; j < 4; ++j) {
+            const float2 v = unpack(g2[i][j]);
+            out[OFF_W2 + (ty + 16 * i) * H + tx + 16 * j] = v.x + v.y;
+        }
+        const float2 v = unpack(g1[i]);
+        out[OFF_W1 + (ty + 16 * i) * F + tx] = v.x + v.y;
     }
     const int k = threadIdx.x;
     out[k < H ? OFF_B1 + k : k < 2 * H ? OFF_B2 + k - H : OFF_W3 + k - 2 * H] = gs;
