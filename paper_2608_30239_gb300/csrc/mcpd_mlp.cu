@@ -36,24 +36,57 @@ constexpr int TR = 64, LD = TR + 4, TB = 256;
 constexpr int SW1 = 0, SB1 = SW1 + F * H, SW2 = SB1 + H, SB2 = SW2 + H * H, SW3 = SB2 + H, SB3 = SW3 + O * H,
               SPARAM = (SB3 + O + 3) / 4 * 4;                    // floats; W1 and W2 stored [in][out]
 
-// Parameters to shared memory in fp32, W1 and W2 transposed to [in][out].
-__device__ __forceinline__ void stage_params(const __nv_bfloat16 *W, float *sW) {
-    for (int i = threadIdx.x; i < NPARAM; i += TB) {
-        int at;
-        if (i < OFF_B1) at = SW1 + (i % F) * H + i / F;
-        else if (i < OFF_W2) at = SB1 + i - OFF_B1;
-        else if (i < OFF_B2) at = SW2 + ((i - OFF_W2) % H) * H + (i - OFF_W2) / H;
-        else at = SB2 + i - OFF_B2;
-        sW[at] = __bfloat162float(W[i]);
+// Parameters to shared memory in fp32, W1 and W2 transposed to [in][out].  A thread loads 8 inputs of an
+// output, a warp 32 outputs of them, so that the transposed stores are conflict-free and all loads are
+// in flight at once, and rows one tile ahead (one parameter at a time, in the order of W, and rows when
+// their tile comes: 50 rows 10.8 us forward and 20.6 backward against 7.8 and 16.5, 83,072 rows 37.0 and 94.3
+// against 29.7 and 89.2).
+__device__ __forceinline__ void load8(const __nv_bfloat16 *W, bool wide, float (&v)[8]) {
+    if (wide) {
+        const uint4 q = __ldg(reinterpret_cast<const uint4 *>(W));
+        const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            v[2 * u] = __uint_as_float(w[u] << 16);
+            v[2 * u + 1] = __uint_as_float(w[u] & 0xFFFF0000u);
+        }
+    } else {                              // the caller's array need only hold bf16
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = __bfloat162float(W[u]);
     }
 }
-
-// Rows r0 .. of X to sX [feature][row]; zeros past n.
-__device__ __forceinline__ void stage_rows(long long n, long long r0, const float *X, float *sX) {
-    for (int i = threadIdx.x; i < TR * F; i += TB) {
-        const long long r = r0 + i / F;
-        sX[(i % F) * LD + i / F] = r < n ? X[r * F + i % F] : 0.f;
+__device__ __forceinline__ void stage_params(const __nv_bfloat16 *W, float *sW) {
+    static_assert(OFF_W1 % 8 == 0 && OFF_W2 % 8 == 0 && H * F / 8 <= TB && H * H / 8 == 2 * TB, "load8 per thread");
+    const bool wide = (reinterpret_cast<uintptr_t>(W) & 15u) == 0;
+    const int t = threadIdx.x, out = t % H, in = t / H * 8;
+    float a[8], b[8], c[8] = {};
+    load8(W + OFF_W2 + out * H + in, wide, a);
+    load8(W + OFF_W2 + out * H + in + TB / H * 8, wide, b);
+    if (t < H * F / 8) load8(W + OFF_W1 + out * F + in, wide, c);
+    const float b1 = __bfloat162float(W[OFF_B1 + t % H]), rest = __bfloat162float(W[OFF_B2 + min(t, NPARAM - OFF_B2 - 1)]);
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+        sW[SW2 + (in + u) * H + out] = a[u];
+        sW[SW2 + (in + TB / H * 8 + u) * H + out] = b[u];
+        if (t < H * F / 8) sW[SW1 + (in + u) * H + out] = c[u];
     }
+    if (t < H) sW[SB1 + t] = b1;
+    if (t < NPARAM - OFF_B2) sW[SB2 + t] = rest;
+}
+
+// Rows r0 .. r0 + 63 of X to sX [feature][row]; zeros past n.  A thread holds 4 features of a row, loaded
+// while the tile before is worked.
+__device__ __forceinline__ float4 load_rows(long long n, long long r0, const float *X, bool wide) {
+    const long long r = r0 + threadIdx.x / 4;
+    const float *const p = X + r * F + threadIdx.x % 4 * 4;
+    if (r >= n) return make_float4(0.f, 0.f, 0.f, 0.f);
+    if (wide) return *reinterpret_cast<const float4 *>(p);
+    return make_float4(p[0], p[1], p[2], p[3]);
+}
+__device__ __forceinline__ void stage_rows(const float4 &v, float *sX) {
+    static_assert(TR * F == 4 * TB, "four values per thread");
+    float *const at = sX + threadIdx.x % 4 * 4 * LD + threadIdx.x / 4;
+    at[0] = v.x; at[LD] = v.y; at[2 * LD] = v.z; at[3 * LD] = v.w;
 }
 
 // Two fp32 values in a register pair; fma2 is an fmaf of each (one instruction issues both).  The gradient's
@@ -122,9 +155,13 @@ __global__ void __launch_bounds__(TB) mlp_forward_kernel(long long n, const floa
     stage_params(W, sW);
     const int c0 = (threadIdx.x & 15) * 4, r0 = (threadIdx.x >> 4) * 4;
     const auto relu = [](float v, int, int) { return fmaxf(v, 0.f); };
-    for (long long row = static_cast<long long>(blockIdx.x) * TR; row < n; row += static_cast<long long>(gridDim.x) * TR) {
+    const bool wide = (reinterpret_cast<uintptr_t>(X) & 15u) == 0;
+    const long long first = static_cast<long long>(blockIdx.x) * TR, stride = static_cast<long long>(gridDim.x) * TR;
+    float4 x = load_rows(n, first, X, wide);
+    for (long long row = first; row < n; row += stride) {
         __syncthreads();
-        stage_rows(n, row, X, sX);
+        stage_rows(x, sX);
+        x = load_rows(n, row + stride, X, wide);
         __syncthreads();
         float acc[4][4];
         tile_gemm<F>(sX, sW + SW1, sW + SB1, r0, c0, acc);
@@ -164,19 +201,29 @@ __global__ void __launch_bounds__(TB) mlp_backward_kernel(long long n, long long
     float *sW = sm, *sW2 = sW + SPARAM, *sX = sW2 + H * H, *sH1 = sX + F * LD, *sH2 = sH1 + H * LD,
           *sD2 = sH2 + H * LD, *sD1 = sD2 + H * LD, *sO = sD1 + H * LD;
     stage_params(W, sW);
-    for (int i = threadIdx.x; i < H * H; i += TB) sW2[i] = __bfloat162float(W[OFF_W2 + i]);   // [out][in]
+    {
+        float v[H * H / TB];
+#pragma unroll
+        for (int i = 0; i < H * H / TB; ++i) v[i] = __bfloat162float(W[OFF_W2 + threadIdx.x + i * TB]);
+#pragma unroll
+        for (int i = 0; i < H * H / TB; ++i) sW2[threadIdx.x + i * TB] = v[i];                   // [out][in]
+    }
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4, c0 = tx * 4, r0 = ty * 4;
     const auto relu = [](float v, int, int) { return fmaxf(v, 0.f); };
     f2 g2[4][4] = {}, g1[4] = {};                                 // sums of the even rows and of the odd ones
     float gs = 0.f, g3 = 0.f;
     const long long begin = static_cast<long long>(blockIdx.x) * chunk, end = min(n, begin + chunk);
+    const bool wide = (reinterpret_cast<uintptr_t>(X) & 15u) == 0;
+    const int dr = threadIdx.x / O, dc = threadIdx.x % O;         // sO [output][row]; zeros past the end
+    auto load_d = [&](long long row) { return threadIdx.x < TR * O && row + dr < end ? dOut[(row + dr) * O + dc] : 0.f; };
+    float4 xn = load_rows(end, begin, X, wide);
+    float dn = load_d(begin);
     for (long long row = begin; row < end; row += TR) {
         __syncthreads();
-        stage_rows(end, row, X, sX);
-        if (threadIdx.x < TR * O) {                               // sO [output][row]; zeros past the end
-            const int r = threadIdx.x / O, o = threadIdx.x % O;
-            sO[o * TR + r] = row + r < end ? dOut[(row + r) * O + o] : 0.f;
-        }
+        stage_rows(xn, sX);
+        if (threadIdx.x < TR * O) sO[dc * TR + dr] = dn;
+        xn = load_rows(end, row + TR, X, wide);
+        dn = load_d(row + TR);
         __syncthreads();
         float acc[4][4];
         tile_gemm<F>(sX, sW + SW1, sW + SB1, r0, c0, acc);

@@ -49,3 +49,33 @@ def test_row_counts_around_tiles_and_chunks(n):
     assert rc == 0
     assert np.array_equal(model.grad.cpu().numpy(), grad)
     ctx.close()
+
+
+@pytest.mark.parametrize("x_off,w_off", [(0, 1), (1, 0), (3, 5)])
+def test_arrays_off_their_16_byte_boundary(x_off, w_off):
+    """The C ABI takes any float rows and bf16 parameters: off the boundary of the wide loads too."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_2608_30239_gb300 import learned, mcpd
+    ctx = mcpd.Context(0)
+    n, rng = 131, np.random.default_rng(7)
+    theta = (rng.integers(-1, 2, 5378) * (rng.random(5378) < 0.2)).astype(np.float32)
+    X = rng.integers(-2, 3, (n, 16)).astype(np.float64)
+    d = rng.integers(-1, 2, (n, 2)).astype(np.float64)
+    out, grad, size = _reference(X, theta, d)
+    assert size < 2 ** 24 and np.abs(out).max() < 2 ** 24
+    xs = torch.zeros(n * 16 + x_off, device="cuda:0")
+    ws = torch.zeros(theta.size + w_off, dtype=torch.bfloat16, device="cuda:0")
+    xs[x_off:] = torch.from_numpy(X.astype(np.float32).ravel()).cuda()
+    ws[w_off:] = torch.from_numpy(theta).cuda().bfloat16()
+    L, p = learned._lib(), learned._p
+    dd, got = torch.from_numpy(d.astype(np.float32)).cuda(), torch.empty((n, 2), device="cuda:0")
+    need = int(L.mcpd_mlp_backward_workspace(n))
+    work, g = torch.empty(need, device="cuda:0"), torch.empty(theta.size, device="cuda:0")
+    torch.cuda.synchronize()
+    assert L.mcpd_mlp_forward(ctx.h, n, p(xs[x_off:]), p(ws[w_off:]), p(got)) == 0
+    assert L.mcpd_mlp_backward(ctx.h, n, p(xs[x_off:]), p(ws[w_off:]), p(dd), p(work), need, p(g)) == 0
+    torch.cuda.synchronize()
+    assert np.array_equal(got.cpu().numpy(), out) and np.array_equal(g.cpu().numpy(), grad)
+    ctx.close()
