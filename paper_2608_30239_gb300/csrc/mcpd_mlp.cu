@@ -146,6 +146,13 @@ __device__ __forceinline__ void tile_store(float *out, int r0, int c0, const flo
             make_float4(f(acc[0][j], 0, j), f(acc[1][j], 1, j), f(acc[2][j], 2, j), f(acc[3][j], 3, j));
 }
 
+// A thread's place in a 16 x 16 grid of 4 x 4 blocks: a warp takes 8 by 4 of them, so that a 16-byte load or
+// store of 8 lanes is one run of 128 bytes along the fast side and 4 addresses along the other.  (A warp of
+// 16 by 2 took 3 wavefronts for the two loads of a product against 2, and its stores conflicted 4-fold: 83,072
+// rows 29.7 us forward and 88.2 backward against 26.6 and 82.0.)
+__device__ __forceinline__ int fast_side() { return (threadIdx.x & 7) + (threadIdx.x >> 5 & 1) * 8; }
+__device__ __forceinline__ int slow_side() { return (threadIdx.x >> 3 & 3) + (threadIdx.x >> 6) * 4; }
+
 constexpr int FWD_SMEM = (SPARAM + (F + 2 * H) * LD) * 4;
 
 // H1 = relu(W1 x + b1), H2 = relu(W2 H1 + b2), out = W3 H2 + b3.
@@ -153,7 +160,7 @@ __global__ void __launch_bounds__(TB) mlp_forward_kernel(long long n, const floa
     extern __shared__ __align__(16) float sm[];
     float *sW = sm, *sX = sW + SPARAM, *sH1 = sX + F * LD, *sH2 = sH1 + H * LD;
     stage_params(W, sW);
-    const int c0 = (threadIdx.x & 15) * 4, r0 = (threadIdx.x >> 4) * 4;
+    const int c0 = slow_side() * 4, r0 = fast_side() * 4;
     const auto relu = [](float v, int, int) { return fmaxf(v, 0.f); };
     const bool wide = (reinterpret_cast<uintptr_t>(X) & 15u) == 0;
     const long long first = static_cast<long long>(blockIdx.x) * TR, stride = static_cast<long long>(gridDim.x) * TR;
@@ -208,7 +215,7 @@ __global__ void __launch_bounds__(TB) mlp_backward_kernel(long long n, long long
 #pragma unroll
         for (int i = 0; i < H * H / TB; ++i) sW2[threadIdx.x + i * TB] = v[i];                   // [out][in]
     }
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4, c0 = tx * 4, r0 = ty * 4;
+    const int tx = fast_side(), ty = slow_side(), c0 = ty * 4, r0 = tx * 4;
     const auto relu = [](float v, int, int) { return fmaxf(v, 0.f); };
     f2 g2[4][4] = {}, g1[4] = {};                                 // sums of the even rows and of the odd ones
     float gs = 0.f, g3 = 0.f;
@@ -237,7 +244,12 @@ __global__ void __launch_bounds__(TB) mlp_backward_kernel(long long n, long long
         });
         __syncthreads();
         tile_gemm<H>(sD2, sW2, nullptr, r0, c0, acc);
-        tile_store(sD1, r0, c0, acc, [&](float v, int i, int j) { return sH1[(c0 + j) * LD + r0 + i] > 0.f ? v : 0.f; });
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const float4 h = *reinterpret_cast<const float4 *>(sH1 + (c0 + j) * LD + r0);
+            *reinterpret_cast<float4 *>(sD1 + (c0 + j) * LD + r0) =
+                make_float4(h.x > 0.f ? acc[0][j] : 0.f, h.y > 0.f ? acc[1][j] : 0.f, h.z > 0.f ? acc[2][j] : 0.f, h.w > 0.f ? acc[3][j] : 0.f);
+        }
         __syncthreads();
 #pragma unroll 2
         for (int r = 0; r < TR; r += 4) {
