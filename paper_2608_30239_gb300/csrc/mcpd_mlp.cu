@@ -202,7 +202,8 @@ constexpr int BWD_SMEM = (SPARAM + H * H + (F + 4 * H) * LD + 2 * TR) * 4;
 
 // Partial parameter gradients of one chunk of rows: the activations recomputed, dOut back-propagated
 // to dZ2 and dZ1, and gW1 = dZ1^T X, gb1 = sum dZ1, gW2 = dZ2^T H1, gb2 = sum dZ2, gW3 = dOut^T H2,
-// gb3 = sum dOut summed over the chunk's rows in registers, in row order; nothing per row goes to
+// gb3 = sum dOut summed over the chunk's rows in registers, in row order (gW1 and gW2 the even and the
+// odd rows apart); nothing per row goes to
 // memory.  A thread owns 16 entries of gW2 and 4 of gW1 (features 16 apart: conflict-free loads), and
 // one of gb1, gb2 or gW3; two warps take gb3.
 __global__ void __launch_bounds__(TB) mlp_backward_kernel(long long n, long long tiles, const float *X, const __nv_bfloat16 *W,
