@@ -421,6 +421,14 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
                 k0 = static_cast<uint32_t>(d.seed); k1 = static_cast<uint32_t>(d.seed >> 32);
                 derive();
                 if (DEG == 0) st[v_dwi() * 32] = v_dw();
+                // Phase 1 steps every lane, those that have found no slot too (a chunk of fewer than
+                // 16), and a step loads by the site drawn ahead: no site of the last chunk's
+                // instance, which may have more clones, is carried over.
+                if constexpr (COUPLED) {
+                    I_cur = col_next = coin_next = 0u;
+                    e_next = 0ull;                      // draws site 0
+                    row_cur = rowAt(0u);
+                }
                 const long long P = v_P(), units = d.units, per = (P + units - 1) / units;
                 first = static_cast<uint32_t>((u - d.unit_begin) * per);
                 cnt = static_cast<uint32_t>(min(per, P - static_cast<long long>(first)));

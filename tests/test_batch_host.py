@@ -1,0 +1,127 @@
+"""A batch's launches as the library's host code makes them, on the stand-in runtime of
+tests/fake_cuda (no GPU): every slot lies in exactly one chunk, no chunk exceeds the bank its
+scratch is laid out for, none is empty, and the scratch holds every warp's part."""
+import ctypes as C
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+import synth
+from paper_2608_30239_gb300 import build, mcpd
+from test_gpu_batch_chunks import CASES, small_chunks
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+PAIR_STATS = 10
+
+
+class Host:
+    def __init__(self, lib):
+        self.lib = lib
+        for name, res, args in (("fake_budget", None, [C.c_int64]), ("fake_live", C.c_int64, []),
+                                ("fake_device", C.c_int, [C.c_int]), ("fake_clear_log", None, []),
+                                ("fake_log", C.c_int64, [C.c_void_p, C.c_int64])):
+            f = getattr(lib, name)
+            f.restype, f.argtypes = res, args
+        self.ctx = mcpd.Context(0, stream=1)
+
+    def run(self, batch, call="mcpd_batch_run_async", *args):
+        """Status, and the launches: dicts of what each was given."""
+        out = np.zeros(max(1, batch.total_active))
+        self.lib.fake_clear_log()
+        p = out.ctypes.data
+        rc = getattr(mcpd.lib(), call)(self.ctx.h, batch.h, *args, p, p)
+        return rc, self.launches()
+
+    def launches(self):
+        n = self.lib.fake_log(None, 0)
+        v = np.zeros(max(n, 1), np.int64)
+        self.lib.fake_log(v.ctypes.data, n)
+        got, at = [], 0
+        while at < n:
+            d = dict(zip(("lanes", "grid", "warps", "bank", "units", "n_inst", "words"), v[at:at + 7].tolist()))
+            d["inst"] = v[at + 7:at + 7 + 4 * d["n_inst"]].reshape(-1, 4)       # slots, first chunk, chunks, clones
+            at += 7 + 4 * d["n_inst"]
+            got.append(d)
+        return got
+
+
+@pytest.fixture(scope="module")
+def host(tmp_path_factory):
+    out = str(tmp_path_factory.mktemp("fake") / "libmcpd_fake.so")
+    inc = ["-I" + build.INCLUDE, "-I" + build.SRC, "-I" + os.path.join(build._cuda_home(), "include")]
+    subprocess.check_call(["g++", "-std=c++17", "-O1", "-fPIC", "-shared", "-ffp-contract=off", "-Wl,-Bsymbolic"] + inc +
+                          [os.path.join(build.SRC, "mcpd_api.cpp"), os.path.join(build.SRC, "mcpd_tables.cpp"),
+                           os.path.join(HERE, "fake_cuda", "fake_cuda.cpp"), "-o", out, "-ldl"])
+    kept = mcpd._lib, build.LIB
+    mcpd._lib, build.LIB = None, out
+    h = Host(mcpd.lib())
+    yield h
+    h.ctx.close()
+    mcpd._lib, build.LIB = kept
+
+
+def warp_words(bank, na):
+    return bank * na + bank + 32 * PAIR_STATS + min(bank, 16) * na          # coupled
+
+
+def check(launches, slots):
+    """Chunks as the kernel cuts them (chunk u of an instance starts at slot u * per)."""
+    total = 0
+    for d in launches:
+        na = int(d["inst"][:, 3].max())
+        assert d["grid"] * d["warps"] * warp_words(d["bank"], na) <= d["words"]
+        at = 0
+        for P, begin, units, _ in d["inst"].tolist():
+            assert begin == at
+            at += units
+            if P == 0:
+                assert units == 0
+                continue
+            per = -(-P // units)
+            assert 0 < per <= d["bank"] and (units - 1) * per < P <= units * per
+            total += P
+        assert at == d["units"]
+    assert total == slots
+
+
+@pytest.mark.parametrize("name", list(CASES))
+def test_more_small_chunks_than_resident_warps(host, name):
+    """The batches of tests/test_gpu_batch_chunks.py: on 152 SMs every chunk is smaller than 16 slots,
+    more chunks than warps are launched, and the later ones belong to smaller instances."""
+    insts, ps = small_chunks(name)
+    b = mcpd.Batch(host.ctx, insts, ps, order_mode=1, classes=1)
+    rc, got = host.run(b)
+    assert rc == 0 and len(got) == 1
+    check(got, sum(kw["slots"] for kw in ps))
+    d = got[0]
+    warps = d["grid"] * d["warps"]
+    first_of = np.searchsorted(d["inst"][:, 1], np.arange(d["units"]), side="right") - 1
+    clones = d["inst"][first_of, 3]
+    assert d["bank"] < 16 and d["units"] > warps == 2432
+    assert clones[warps:].max() < clones[:warps].max()
+    b.close()
+
+
+@pytest.mark.parametrize("classes", [0, 1, 3])
+@pytest.mark.parametrize("slots", [1, 7, 33, 512, 1000])
+def test_every_slot_in_one_chunk(host, slots, classes):
+    rng = np.random.default_rng(slots)
+    insts = [synth.make_instance(int(n), int(n) // 13, 4 + i % 5, 2, 0.05, 0.1, 2 / n, i, 50 + i)
+             for i, n in enumerate(rng.integers(200, 4000, 24))]
+    ps = [dict(slots=slots + i % 3, horizon=2 * inst.n, seed=i, instance_id=i) for i, inst in enumerate(insts)]
+    b = mcpd.Batch(host.ctx, insts, ps, classes=classes)
+    want = sum(kw["slots"] for kw in ps)
+    rc, got = host.run(b)
+    assert rc == 0
+    check(got, want)
+    mask = np.array([i % 2 for i in range(len(insts))], np.int32)
+    rc, got = host.run(b, "mcpd_batch_extend_async", mask.ctypes.data)
+    assert rc == 0
+    check(got, sum(kw["slots"] for kw, m in zip(ps, mask) if m))
+    b.set_shape(warps_per_block=3)
+    rc, got = host.run(b)
+    assert rc == 0
+    check(got, want)
+    b.close()
