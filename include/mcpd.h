@@ -270,7 +270,9 @@ int mcpd_batch_offsets(const mcpd_batch *batch, int64_t *offsets);
 /* Choose the launch shape of every class: lanes per pair (1: the sampling kernel; 8, 16 or 32: a
  * lane group per pair, coupled batches only; all give identical results) and at most
  * warps_per_block warps per block (0: as many as the kernel and the class's largest pair state
- * allow).  May reallocate the per-pair scratch; invalidates a captured graph. */
+ * allow).  May reallocate the per-pair scratch; invalidates a captured graph.  On failure the batch
+ * keeps the shape it had; only if its scratch cannot be allocated again has it none, and runs return
+ * MCPD_ENOMEM until a shape is set. */
 int mcpd_batch_set_shape(mcpd_ctx *ctx, mcpd_batch *batch, int32_t lanes_per_pair,
                          int32_t warps_per_block);
 /* Enqueue one decode of every instance; est_dev, se_dev: device arrays [info[0]]. */

@@ -62,6 +62,7 @@ int set_err(mcpd_ctx *ctx, int code, const std::string &msg) {
 
 int cu_status(mcpd_ctx *ctx, cudaError_t e, const char *what) {
     if (e == cudaSuccess) return MCPD_OK;
+    cudaGetLastError();              // reported here: the next launch must not find it
     return set_err(ctx, e == cudaErrorMemoryAllocation ? MCPD_ENOMEM : MCPD_ECUDA,
                    std::string(what) + ": " + cudaGetErrorString(e));
 }
@@ -616,6 +617,7 @@ struct mcpd_batch {
     int n_classes = 0;
     int32_t n_inst = 0, lanes = 1;
     bool coupled = true;
+    bool shaped = false;                   // every launch has its shape, chunks and scratch
     mcpd::InstDesc *d_insts = nullptr;
     std::vector<mcpd::InstDesc> insts;     // in launch order, as the device holds them
     std::vector<mcpd::InstDesc> insts0;    // the descriptors of a decode from the first slot
@@ -673,17 +675,46 @@ void number_units(mcpd_batch *b, std::vector<mcpd::InstDesc> &insts) {
     }
 }
 
+// Give the launches the shapes of `shapes` (copies of b->cls): the scratch each holds stays with it and
+// is replaced where the shape needs more.
+int hold_shapes(mcpd_ctx *ctx, mcpd_batch *b, const std::vector<BatchClass> &shapes) {
+    for (size_t ci = 0; ci < b->cls.size(); ++ci) {
+        BatchClass to = shapes[ci], &c = b->cls[ci];
+        to.scratch = c.scratch;
+        to.scratch_held = c.scratch_held;
+        to.bp.pair_scratch = c.bp.pair_scratch;
+        c = to;
+    }
+    for (BatchClass &c : b->cls) {
+        if (c.scratch_words <= c.scratch_held) continue;
+        free_list(c.scratch);
+        c.scratch_held = 0;
+        const int rc = balloc(ctx, c.scratch, &c.bp.pair_scratch, c.scratch_words);
+        if (rc != MCPD_OK) return rc;
+        c.scratch_held = c.scratch_words;
+    }
+    return MCPD_OK;
+}
+
+int need_shape(mcpd_ctx *ctx, const mcpd_batch *b) {
+    return b->shaped ? MCPD_OK : set_err(ctx, MCPD_ENOMEM, "the batch has no launch shape: set one that fits the device memory");
+}
+
 // Launch shape of every class: `lanes` per pair (1: the sampling kernel; 8, 16, 32: a lane group
 // per pair) and at most `warps` per block (0: as many as fit the class's largest pair state),
-// the chunks, and the scratch it needs.
+// the chunks, and the scratch it needs.  If that fails, the batch keeps the shape it had (without a
+// captured graph if its scratch moved), or, if not even that one's scratch can be had again, has none
+// until a later call gives it one.
 int batch_shape(mcpd_ctx *ctx, mcpd_batch *b, int warps, int lanes = 1) {
     if (lanes != 1 && lanes != 8 && lanes != 16 && lanes != 32)
         return set_err(ctx, MCPD_EINVAL, "lanes per pair must be 1, 8, 16 or 32");
     if (lanes > 1 && !b->coupled) return set_err(ctx, MCPD_EINVAL, "lane groups run coupled batches only");
+    const std::vector<BatchClass> before = b->cls;
+    std::vector<BatchClass> shapes = before;
     double work = 0.0;                 // columns x words of all classes: what they share the GPU by
-    for (const BatchClass &c : b->cls) work += static_cast<double>(b->total_work0[&c - b->cls.data()]) * c.bp.max_wpp;
-    for (size_t ci = 0; ci < b->cls.size(); ++ci) {
-        BatchClass &c = b->cls[ci];
+    for (size_t ci = 0; ci < shapes.size(); ++ci) work += static_cast<double>(b->total_work0[ci]) * shapes[ci].bp.max_wpp;
+    for (size_t ci = 0; ci < shapes.size(); ++ci) {
+        BatchClass &c = shapes[ci];
         const long long class_slots = b->total_work0[ci];
         int per_sm = 1, w = 0;
         if (lanes == 1) {
@@ -739,24 +770,26 @@ int batch_shape(mcpd_ctx *ctx, mcpd_batch *b, int warps, int lanes = 1) {
         c.warps = w;
         c.block = w * 32;
         c.bp.lanes = lanes;
-        if (c.scratch_words > c.scratch_held) {
-            free_list(c.scratch);
-            c.scratch_held = 0;
-            const int rc = balloc(ctx, c.scratch, &c.bp.pair_scratch, c.scratch_words);
-            if (rc != MCPD_OK) return rc;
-            c.scratch_held = c.scratch_words;
-        }
     }
+    if (b->graph_exec) { cudaGraphExecDestroy(b->graph_exec); b->graph_exec = nullptr; }
+    if (b->graph) { cudaGraphDestroy(b->graph); b->graph = nullptr; }
     // The kernels lay the scratch out by their shape, so a run in another shape starts from a
     // cleared one; the chunks are the descriptors' too.
     b->dirty = true;
+    const bool had = b->shaped;
+    b->shaped = false;
+    const int rc = hold_shapes(ctx, b, shapes);
+    if (rc != MCPD_OK) {
+        const std::string why = ctx->err;
+        if (had && hold_shapes(ctx, b, before) == MCPD_OK) b->shaped = true;
+        return set_err(ctx, rc, why);
+    }
     number_units(b, b->insts0);
     number_units(b, b->insts);
     CU(cudaMemcpyAsync(b->d_insts, b->insts.data(), sizeof(mcpd::InstDesc) * b->insts.size(), cudaMemcpyHostToDevice,
                        ctx->stream));
     b->lanes = lanes;
-    if (b->graph_exec) { cudaGraphExecDestroy(b->graph_exec); b->graph_exec = nullptr; }
-    if (b->graph) { cudaGraphDestroy(b->graph); b->graph = nullptr; }
+    b->shaped = true;
     return MCPD_OK;
 }
 
@@ -1034,9 +1067,10 @@ int mcpd_batch_set_shape(mcpd_ctx *ctx, mcpd_batch *b, int32_t lanes_per_pair, i
 int mcpd_batch_run_async(mcpd_ctx *ctx, mcpd_batch *b, double *est_dev, double *se_dev) {
     NvtxRange nvtx_range("mcpd.batch_run");
     if (!ctx || !b || !est_dev || !se_dev) return MCPD_EINVAL;
-    CU(cudaSetDevice(ctx->device));
-    int rc = restore_descriptors(ctx, b);
+    int rc = need_shape(ctx, b);
     if (rc != MCPD_OK) return rc;
+    CU(cudaSetDevice(ctx->device));
+    if ((rc = restore_descriptors(ctx, b)) != MCPD_OK) return rc;
     CU(cudaEventRecord(b->ev0, ctx->stream));
     rc = batch_enqueue(ctx, b, est_dev, se_dev, false);
     if (rc != MCPD_OK) return rc;
@@ -1050,6 +1084,7 @@ int mcpd_batch_extend_async(mcpd_ctx *ctx, mcpd_batch *b, const int32_t *mask, d
     NvtxRange nvtx_range("mcpd.batch_extend");
     if (!ctx || !b || !est_dev || !se_dev) return MCPD_EINVAL;
     if (!b->ran) return set_err(ctx, MCPD_EINVAL, "nothing to extend: run the batch first");
+    if (need_shape(ctx, b) != MCPD_OK) return MCPD_ENOMEM;
     CU(cudaSetDevice(ctx->device));
     // Each chosen instance runs its next P_i slots (the next global ids after those in its
     // buckets); the others run none.  Work items are renumbered per class.
@@ -1087,6 +1122,7 @@ int mcpd_batch_extend_async(mcpd_ctx *ctx, mcpd_batch *b, const int32_t *mask, d
 int mcpd_batch_capture_graph(mcpd_ctx *ctx, mcpd_batch *b, double *est_dev, double *se_dev) {
     NvtxRange nvtx_range("mcpd.batch_capture_graph");
     if (!ctx || !b || !est_dev || !se_dev) return MCPD_EINVAL;
+    if (need_shape(ctx, b) != MCPD_OK) return MCPD_ENOMEM;
     CU(cudaSetDevice(ctx->device));
     if (!ctx->stream) return set_err(ctx, MCPD_EINVAL, "graph capture needs a non-default stream");
     {

@@ -15,6 +15,7 @@
 
 namespace {
 size_t g_budget = size_t(1) << 40, g_live = 0;
+long long g_allocs_left = -1;          // allocations that succeed before all fail (-1: no limit)
 int g_device = 0;
 cudaError_t g_last = cudaSuccess;
 std::map<char *, size_t> g_blocks;
@@ -33,6 +34,7 @@ size_t room_at(const void *p) {
 
 extern "C" {
 void fake_budget(long long bytes) { g_budget = static_cast<size_t>(bytes); }
+void fake_allocs(long long left) { g_allocs_left = left; }
 long long fake_live() { return static_cast<long long>(g_live); }
 int fake_device(int set) { if (set >= 0) g_device = set; return g_device; }
 long long fake_log(long long *out, long long cap) {
@@ -43,7 +45,8 @@ long long fake_log(long long *out, long long cap) {
 void fake_clear_log() { g_log.clear(); }
 
 cudaError_t cudaMalloc(void **p, size_t bytes) {
-    if (g_live + bytes > g_budget) return g_last = cudaErrorMemoryAllocation;
+    if (g_live + bytes > g_budget || g_allocs_left == 0) return g_last = cudaErrorMemoryAllocation;
+    if (g_allocs_left > 0) --g_allocs_left;
     char *c = static_cast<char *>(std::malloc(bytes ? bytes : 1));   // pages are taken only where they are touched
     if (!c) return g_last = cudaErrorMemoryAllocation;
     g_blocks[c] = bytes;

@@ -19,7 +19,8 @@ PAIR_STATS = 10
 class Host:
     def __init__(self, lib):
         self.lib = lib
-        for name, res, args in (("fake_budget", None, [C.c_int64]), ("fake_live", C.c_int64, []),
+        for name, res, args in (("fake_budget", None, [C.c_int64]), ("fake_allocs", None, [C.c_int64]),
+                                ("fake_live", C.c_int64, []),
                                 ("fake_device", C.c_int, [C.c_int]), ("fake_clear_log", None, []),
                                 ("fake_log", C.c_int64, [C.c_void_p, C.c_int64])):
             f = getattr(lib, name)
@@ -124,4 +125,65 @@ def test_every_slot_in_one_chunk(host, slots, classes):
     rc, got = host.run(b)
     assert rc == 0
     check(got, want)
+    b.close()
+
+
+def _growing(host):
+    """Two launches whose scratch grows from 16 warps per block (chunks of 37 slots) to 9 (of 32)."""
+    insts = [synth.make_instance(900, 60, 4, 2, 0.05, 0.1, 0.003, i, 50 + i) for i in range(16)]
+    ps = [dict(slots=5526, horizon=2 * inst.n, seed=i, instance_id=i) for i, inst in enumerate(insts)]
+    b = mcpd.Batch(host.ctx, insts, ps, classes=2)
+    rc, got = host.run(b)
+    assert rc == 0 and [(d["bank"], d["warps"]) for d in got] == [(37, 16), (37, 16)]
+    return b, sum(kw["slots"] for kw in ps)
+
+
+def _set_shape(host, b, lanes, warps):
+    return mcpd.lib().mcpd_batch_set_shape(host.ctx.h, b.h, lanes, warps)
+
+
+@pytest.mark.parametrize("left", [0, 1, 2])
+def test_failed_shape_change(host, left):
+    """Memory runs out at the first or the second of two launches, and for good (with two
+    allocations the change succeeds): the batch refuses to run, and its graph is gone, until a
+    shape is set."""
+    b, slots = _growing(host)
+    assert host.run(b, "mcpd_batch_capture_graph")[0] == 0
+    host.lib.fake_allocs(left)
+    try:
+        want = 0 if left == 2 else mcpd.MCPD_ENOMEM
+        assert _set_shape(host, b, 1, 9) == want
+        assert mcpd.lib().mcpd_batch_launch_graph(host.ctx.h, b.h) == mcpd.MCPD_EINVAL
+        for call, args in (("mcpd_batch_run_async", ()), ("mcpd_batch_extend_async", (None,)), ("mcpd_batch_capture_graph", ())):
+            rc, got = host.run(b, call, *args)
+            assert rc == want
+            if rc == 0:
+                check(got, slots)
+    finally:
+        host.lib.fake_allocs(-1)
+    b.set_shape(9)
+    rc, got = host.run(b)
+    assert rc == 0 and [(d["bank"], d["warps"]) for d in got] == [(32, 9), (32, 9)]
+    check(got, slots)
+    b.close()
+
+
+def test_failed_shape_change_keeps_the_shape(host):
+    """Memory for the first launch's larger scratch only: the batch goes on in the shape it had, and
+    its launches find no error left over."""
+    b, slots = _growing(host)
+    words = [d["words"] for d in host.run(b)[1]]
+    host.lib.fake_budget(host.lib.fake_live() + 8 * words[0] * 4 // 100)        # each grows by 3.3%
+    try:
+        assert _set_shape(host, b, 1, 9) == mcpd.MCPD_ENOMEM
+        rc, got = host.run(b)
+        assert rc == 0 and [(d["bank"], d["warps"]) for d in got] == [(37, 16), (37, 16)]
+        assert got[0]["words"] > words[0] and got[1]["words"] == words[1]       # the first one did grow
+        check(got, slots)
+        assert _set_shape(host, b, 5, 9) == mcpd.MCPD_EINVAL                     # refused before any change
+        rc, got = host.run(b)
+        assert rc == 0
+        check(got, slots)
+    finally:
+        host.lib.fake_budget(1 << 40)
     b.close()
