@@ -230,6 +230,16 @@ __global__ void __launch_bounds__(TB) mlp_backward_kernel(long long n, long long
     auto load_d = [&](long long row) { return threadIdx.x < TR * O && row + dr < end ? dOut[(row + dr) * O + dc] : 0.f; };
     float4 xn = load_rows(end, begin, X, wide);
     float dn = load_d(begin);
+    // The rows past the end have activations too (the biases'); they are no one's rows, and zeros would
+    // not keep an infinite one out of the sums.  A thread clears the entries that it stored.
+    auto clear_past = [&](float *out, long long left) {
+        if (left >= TR) return;
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (r0 + i >= left)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) out[(c0 + j) * LD + r0 + i] = 0.f;
+    };
     for (long long row = begin; row < end; row += TR) {
         __syncthreads();
         stage_rows(xn, sX);
@@ -240,6 +250,7 @@ __global__ void __launch_bounds__(TB) mlp_backward_kernel(long long n, long long
         float acc[4][4];
         tile_gemm<F>(sX, sW + SW1, sW + SB1, r0, c0, acc);
         tile_store(sH1, r0, c0, acc, relu);
+        clear_past(sH1, end - row);
         __syncthreads();
         tile_gemm<H>(sH1, sW + SW2, sW + SB2, r0, c0, acc);
         tile_store(sH2, r0, c0, acc, relu);
@@ -247,6 +258,8 @@ __global__ void __launch_bounds__(TB) mlp_backward_kernel(long long n, long long
             const float dh = fmaf(sW[SW3 + c0 + j], sO[r0 + i], sW[SW3 + H + c0 + j] * sO[TR + r0 + i]);
             return z > 0.f ? dh : 0.f;
         });
+        clear_past(sH2, end - row);
+        clear_past(sD2, end - row);
         __syncthreads();
         tile_gemm<H>(sD2, sW2, nullptr, r0, c0, acc);
 #pragma unroll
