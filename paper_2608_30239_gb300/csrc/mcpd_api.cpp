@@ -294,8 +294,15 @@ int mcpd_plan_create(mcpd_ctx *ctx, const mcpd_design *design, const uint8_t *y,
     const size_t o_nstar = take(slots * 4, 256), o_slot_S = take(slots * 8, 256), o_reps = take(slots * 4, 256);
     const size_t o_trace = take(static_cast<size_t>(pl->n_trace) * t.na * 8, 256);
     const size_t o_rec = take(static_cast<size_t>(pl->n_trace) * t.trace_reps * (4 + t.trace_steps) * 4, 256);
-    const size_t o_scratch = take(pl->scratch_words() * 8, 256);
-    CU_OR(cudaMalloc(&pl->mem, total), mcpd_plan_destroy(pl));
+    // The scratch comes last.  Where the memory does not hold it, smaller chunks, with fewer slots' sums
+    // each, do with less (and take longer: 3 and 5% for chunks of 64 and 32 slots).
+    const size_t o_scratch = take(0, 256);
+    for (;; kp.bank = (kp.bank + 1) / 2) {
+        const cudaError_t e = cudaMalloc(&pl->mem, o_scratch + pl->scratch_words() * 8);
+        if (e == cudaSuccess) break;
+        if (e != cudaErrorMemoryAllocation || kp.bank == 1) CU_OR(e, mcpd_plan_destroy(pl));
+        cudaGetLastError();
+    }
     unsigned char *const mem = static_cast<unsigned char *>(pl->mem);
     std::vector<unsigned char> tab(tables_end);
     auto put = [&](size_t at, const void *src, size_t bytes) { if (bytes) std::memcpy(tab.data() + at, src, bytes); };
@@ -676,14 +683,18 @@ void number_units(mcpd_batch *b, std::vector<mcpd::InstDesc> &insts) {
 }
 
 // Give the launches the shapes of `shapes` (copies of b->cls): the scratch each holds stays with it and
-// is replaced where the shape needs more.
-int hold_shapes(mcpd_ctx *ctx, mcpd_batch *b, const std::vector<BatchClass> &shapes) {
+// is replaced where the shape needs more (`tight`: or less, before any is allocated).
+int hold_shapes(mcpd_ctx *ctx, mcpd_batch *b, const std::vector<BatchClass> &shapes, bool tight = false) {
     for (size_t ci = 0; ci < b->cls.size(); ++ci) {
         BatchClass to = shapes[ci], &c = b->cls[ci];
         to.scratch = c.scratch;
         to.scratch_held = c.scratch_held;
         to.bp.pair_scratch = c.bp.pair_scratch;
         c = to;
+        if (tight && c.scratch_words < c.scratch_held) {
+            free_list(c.scratch);
+            c.scratch_held = 0;
+        }
     }
     for (BatchClass &c : b->cls) {
         if (c.scratch_words <= c.scratch_held) continue;
@@ -778,10 +789,19 @@ int batch_shape(mcpd_ctx *ctx, mcpd_batch *b, int warps, int lanes = 1) {
     b->dirty = true;
     const bool had = b->shaped;
     b->shaped = false;
-    const int rc = hold_shapes(ctx, b, shapes);
+    int rc = hold_shapes(ctx, b, shapes);
+    // Where the memory does not hold the scratch, smaller chunks on the same warps do with less.
+    for (int32_t most = 32; rc == MCPD_ENOMEM && lanes == 1 && most > 0; most /= 2) {
+        for (BatchClass &c : shapes) {
+            c.bp.bank = std::min(c.bp.bank, most);
+            c.pairs = static_cast<long long>(c.grid) * c.warps * c.bp.bank;
+            c.scratch_words = static_cast<size_t>(c.grid) * c.warps * mcpd::warp_words(c.bp.bank, c.bp.max_na, b->coupled);
+        }
+        rc = hold_shapes(ctx, b, shapes, true);
+    }
     if (rc != MCPD_OK) {
         const std::string why = ctx->err;
-        if (had && hold_shapes(ctx, b, before) == MCPD_OK) b->shaped = true;
+        if (had && hold_shapes(ctx, b, before, true) == MCPD_OK) b->shaped = true;
         return set_err(ctx, rc, why);
     }
     number_units(b, b->insts0);

@@ -171,19 +171,84 @@ def test_failed_shape_change(host, left):
 def test_failed_shape_change_keeps_the_shape(host):
     """Memory for the first launch's larger scratch only: the batch goes on in the shape it had, and
     its launches find no error left over."""
-    b, slots = _growing(host)
-    words = [d["words"] for d in host.run(b)[1]]
-    host.lib.fake_budget(host.lib.fake_live() + 8 * words[0] * 4 // 100)        # each grows by 3.3%
+    insts = [synth.make_instance(4000, 100, 4, 2, 0.05, 0.1, 0.003, i, 50 + i) for i in range(8)]
+    slots = 8 * 2432
+    b = mcpd.Batch(host.ctx, insts, [dict(slots=2432, horizon=4000, seed=i, instance_id=i) for i in range(8)], classes=2)
+    rc, got = host.run(b)
+    assert rc == 0
+    words = [d["words"] for d in got]
+    more = 9728 * (2 * 4000 + 125 + PAIR_STATS) - words[0]                      # lane groups of 8, 9728 pairs per launch
+    assert 0 < more < words[0]
+    host.lib.fake_budget(host.lib.fake_live() + 8 * more * 3 // 2)
     try:
-        assert _set_shape(host, b, 1, 9) == mcpd.MCPD_ENOMEM
-        rc, got = host.run(b)
-        assert rc == 0 and [(d["bank"], d["warps"]) for d in got] == [(37, 16), (37, 16)]
-        assert got[0]["words"] > words[0] and got[1]["words"] == words[1]       # the first one did grow
-        check(got, slots)
+        assert _set_shape(host, b, 8, 0) == mcpd.MCPD_ENOMEM
         assert _set_shape(host, b, 5, 9) == mcpd.MCPD_EINVAL                     # refused before any change
-        rc, got = host.run(b)
-        assert rc == 0
-        check(got, slots)
+        rc, again = host.run(b)
+        assert rc == 0 and [(d["lanes"], d["bank"], d["grid"], d["words"]) for d in again] == \
+            [(d["lanes"], d["bank"], d["grid"], d["words"]) for d in got]
+        check(again, slots)
     finally:
         host.lib.fake_budget(1 << 40)
+    b.set_shape(lanes_per_pair=8)
+    assert [d["words"] for d in host.run(b)[1]] == [w + more for w in words]
     b.close()
+
+
+@pytest.mark.parametrize("part", [0.9, 0.4, 0.1])
+def test_batch_in_less_memory(host, part):
+    """Where a batch's scratch does not fit, its chunks get smaller: at creation, and for a shape set
+    later."""
+    insts = [synth.make_instance(n, 60, 4, 2, 0.05, 0.1, 0.003, n, 50 + n) for n in (900, 800, 700, 600)]
+    ps = [dict(slots=30000, horizon=2 * inst.n, seed=i, instance_id=i) for i, inst in enumerate(insts)]
+    base = host.lib.fake_live()
+    b = mcpd.Batch(host.ctx, insts, ps, classes=2)
+    rc, got = host.run(b)
+    bank, need = [d["bank"] for d in got], host.lib.fake_live() - base
+    fixed = need - 8 * sum(d["words"] for d in got)
+    b.close()
+    host.lib.fake_budget(base + fixed + int(part * (need - fixed)))
+    try:
+        b = mcpd.Batch(host.ctx, insts, ps, classes=2)
+        for warps in (0, 7, 0):
+            b.set_shape(warps)
+            rc, got = host.run(b)
+            assert rc == 0
+            check(got, 120000)
+            if warps == 0:
+                assert all(d["bank"] < was for d, was in zip(got, bank))
+        b.close()
+        host.lib.fake_budget(base + fixed)
+        with pytest.raises(mcpd.McpdError, match="ENOMEM"):
+            mcpd.Batch(host.ctx, insts, ps, classes=2)
+    finally:
+        host.lib.fake_budget(1 << 40)
+    assert host.lib.fake_live() == base
+
+
+@pytest.mark.parametrize("part", [1.0, 0.56, 0.3, 0.05])
+def test_plan_in_less_memory(host, part):
+    """A plan whose scratch (some 100 sums of n_a words per warp) does not fit gets smaller chunks, for
+    all that it fits in: 0.56 of it is what one sum pair per lane (64 per warp) would take."""
+    inst = synth.make_instance(1298, 97, 6, 3, 0.1, 0.2, 3 / 1298, 1, 2)
+    base = host.lib.fake_live()
+    kw = dict(slots=524288, horizon=2000, seed=3)
+    plan = mcpd.Plan(host.ctx, inst, **kw)
+    need = host.lib.fake_live() - base
+    plan.close()
+    host.lib.fake_budget(base + int(part * need))
+    try:
+        plan = mcpd.Plan(host.ctx, inst, **kw)
+        out = np.zeros(1298)
+        for call, args in (("mcpd_run_async", ()), ("mcpd_run_slots_async", (1000, 0)), ("mcpd_run_slots_async", (700000, 1))):
+            host.lib.fake_clear_log()
+            assert getattr(mcpd.lib(), call)(host.ctx.h, plan.h, *args, out.ctypes.data, out.ctypes.data) == 0
+            d, = host.launches()
+            assert 0 < d["units"] <= d["bank"]                                   # a plan logs its chunk there
+            assert d["grid"] * d["warps"] * warp_words(d["bank"], 1298) <= d["words"]
+        plan.close()
+        host.lib.fake_budget(base + need // 1000)
+        with pytest.raises(mcpd.McpdError, match="ENOMEM"):
+            mcpd.Plan(host.ctx, inst, **kw)
+    finally:
+        host.lib.fake_budget(1 << 40)
+    assert host.lib.fake_live() == base
