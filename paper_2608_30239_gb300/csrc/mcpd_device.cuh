@@ -79,16 +79,21 @@ static __device__ __noinline__ long long lag_prefix(uint32_t u, uint32_t k, uint
     return static_cast<long long>(m - k + 1u) + F(u - k) - (u > m ? F(u - m - 1u) : 0ll);
 }
 
-// Add G and G^2 (128-bit, carried into the high word) of one slot to bucket N*_p - 1.
-static __device__ __forceinline__ void bucket_add(unsigned long long *S1, unsigned long long *S2lo,
-                                           unsigned long long *S2hi, int na, int bkt, int j, long long g) {
+// Add s1 and the 128-bit s2 = (lo, hi), carried into the high word, to clone j of bucket bkt.
+static __device__ __forceinline__ void bucket_add_sums(unsigned long long *S1, unsigned long long *S2lo,
+                                                unsigned long long *S2hi, int na, int bkt, int j, long long s1,
+                                                unsigned long long lo, unsigned long long hi) {
     const size_t idx = static_cast<size_t>(bkt) * na + j;
-    atomicAdd(&S1[idx], static_cast<unsigned long long>(g));
-    const unsigned long long a = static_cast<unsigned long long>(g < 0 ? -g : g);
-    const unsigned long long lo = a * a, hi = __umul64hi(a, a);
+    atomicAdd(&S1[idx], static_cast<unsigned long long>(s1));
     const unsigned long long old = atomicAdd(&S2lo[idx], lo);
     const unsigned long long carry = (old + lo < old) ? 1ull : 0ull;
     if (hi + carry) atomicAdd(&S2hi[idx], hi + carry);
+}
+// Add G and G^2 of one slot to bucket N*_p - 1.
+static __device__ __forceinline__ void bucket_add(unsigned long long *S1, unsigned long long *S2lo,
+                                           unsigned long long *S2hi, int na, int bkt, int j, long long g) {
+    const unsigned long long a = static_cast<unsigned long long>(g < 0 ? -g : g);
+    bucket_add_sums(S1, S2lo, S2hi, na, bkt, j, g, a * a, __umul64hi(a, a));
 }
 
 }  // namespace mcpd
