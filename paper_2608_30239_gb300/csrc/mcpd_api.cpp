@@ -49,7 +49,7 @@ struct mcpd_plan {
     long long last_pairs = 0;        // pairs the last launch held (its grid x block)
     mutable int64_t h2d_bytes = 0, d2h_bytes = 0;   // bytes copied between host and device (fetches too)
     size_t scratch_words() const {
-        return static_cast<size_t>(grid) * (block / 32) * mcpd::warp_words(kp.bank, t.na, t.coupled);
+        return static_cast<size_t>(grid) * (block / 32) * mcpd::warp_words(kp.bank, t.na, kp.marks, t.coupled);
     }
 };
 
@@ -250,9 +250,10 @@ int mcpd_plan_create(mcpd_ctx *ctx, const mcpd_design *design, const uint8_t *y,
 
     // Launch shape: tables first in shared memory, then one 32-column region per warp.
     const size_t tables = mcpd::kernel_table_bytes(t);
+    const int32_t marks = t.trace_steps > 0 ? 0 : mcpd::mark_words(t.coupled, mcpd::mark_steps(t.coupled, t.B, t.unit, t.lag), t.na, t.na, t.W);
     mcpd::PairsShape shape;
     rc = mcpd::pairs_shape(t.coupled, t.scan, t.udeg, false, tables, t.wpp, ctx->smem_optin, t.P,
-                           ctx->sm_count, 0, t.capped || t.lag > 1, !t.Tnu.empty(), &shape);
+                           ctx->sm_count, 0, t.capped || t.lag > 1, marks > 0, &shape);
     if (rc != MCPD_OK) {
         delete pl;
         return set_err(ctx, rc, rc == MCPD_ETOO_LARGE ? "instance too large for the one-thread-per-pair layout"
@@ -272,6 +273,7 @@ int mcpd_plan_create(mcpd_ctx *ctx, const mcpd_design *design, const uint8_t *y,
         const mcpd::ChunkShape cs = mcpd::chunk_shape(t.P, pl->grid, warps, mcpd::kBank);
         kp.chunk = cs.chunk;
         kp.bank = std::max(32, cs.chunk);         // a later run may bring more slots
+        kp.marks = marks;
     }
     if (t.trace_stride > 0) pl->n_trace = (t.P + t.trace_stride - 1) / t.trace_stride;
     size_t total = 0;
@@ -731,12 +733,12 @@ int batch_shape(mcpd_ctx *ctx, mcpd_batch *b, int warps, int lanes = 1) {
         if (lanes == 1) {
             mcpd::PairsShape shape;
             int rc = mcpd::pairs_shape(c.bp.coupled, c.bp.scan, c.bp.udeg, true, 0, c.bp.max_wpp, ctx->smem_optin, 0,
-                                       ctx->sm_count, 0, c.bp.ext != 0, true, &shape);
+                                       ctx->sm_count, 0, c.bp.ext != 0, c.bp.marks > 0, &shape);
             if (rc == MCPD_ETOO_LARGE) return set_err(ctx, rc, "largest instance does not fit one warp of pair state");
             if (rc != MCPD_OK) return set_err(ctx, rc, "cudaFuncSetAttribute / occupancy");
             if (warps > 0 && warps < shape.warps) {
                 rc = mcpd::pairs_shape(c.bp.coupled, c.bp.scan, c.bp.udeg, true, 0, c.bp.max_wpp, ctx->smem_optin, 0,
-                                       ctx->sm_count, warps, c.bp.ext != 0, true, &shape);
+                                       ctx->sm_count, warps, c.bp.ext != 0, c.bp.marks > 0, &shape);
                 if (rc != MCPD_OK) return set_err(ctx, rc, "launch shape");
             }
             w = shape.warps;
@@ -759,7 +761,7 @@ int batch_shape(mcpd_ctx *ctx, mcpd_batch *b, int warps, int lanes = 1) {
             c.grid = static_cast<int>(std::max<long long>(1, std::min<long long>(static_cast<long long>(ctx->sm_count) * per_sm,
                                                                                   (units + w - 1) / w)));
             c.pairs = static_cast<long long>(c.grid) * w * std::min(32, c.bp.bank);
-            c.scratch_words = static_cast<size_t>(c.grid) * w * mcpd::warp_words(c.bp.bank, c.bp.max_na, b->coupled);
+            c.scratch_words = static_cast<size_t>(c.grid) * w * mcpd::warp_words(c.bp.bank, c.bp.max_na, c.bp.marks, b->coupled);
         } else {
             const size_t per_warp = static_cast<size_t>(32 / lanes) * 2 * c.bp.max_wpp * 4;
             const int cap = mcpd::group_max_threads(lanes) / 32;
@@ -795,7 +797,7 @@ int batch_shape(mcpd_ctx *ctx, mcpd_batch *b, int warps, int lanes = 1) {
         for (BatchClass &c : shapes) {
             c.bp.bank = std::min(c.bp.bank, most);
             c.pairs = static_cast<long long>(c.grid) * c.warps * c.bp.bank;
-            c.scratch_words = static_cast<size_t>(c.grid) * c.warps * mcpd::warp_words(c.bp.bank, c.bp.max_na, b->coupled);
+            c.scratch_words = static_cast<size_t>(c.grid) * c.warps * mcpd::warp_words(c.bp.bank, c.bp.max_na, c.bp.marks, b->coupled);
         }
         rc = hold_shapes(ctx, b, shapes, true);
     }
@@ -1012,6 +1014,13 @@ int mcpd_batch_create(mcpd_ctx *ctx, int32_t n_inst, const mcpd_design *designs,
         bp.coupled = b->coupled ? 1 : 0;
         bp.scan = b->t[0].scan;
         bp.lanes = 1;
+        double steps = 0.0, clones = 0.0;
+        for (int32_t k = 0; k < b->cls[c].count; ++k) {
+            const mcpd::InstDesc &d = b->insts[static_cast<size_t>(b->cls[c].first) + k];
+            steps += static_cast<double>(d.P) * mcpd::mark_steps(b->coupled, d.B, d.unit, d.lag);
+            clones += static_cast<double>(d.P) * d.na;
+        }
+        bp.marks = mcpd::mark_words(b->coupled, steps, clones, bp.max_na, bp.max_W);
         bp.counters = b->d_counters + static_cast<size_t>(c) * mcpd::kNumCounters;
         bp.error = b->d_error;
     }

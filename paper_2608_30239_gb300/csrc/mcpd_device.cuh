@@ -61,6 +61,9 @@ static __device__ __noinline__ uint32_t philox_low_word(uint4 c, uint32_t k0, ui
 static __device__ __forceinline__ void red_add(long long *a, long long v) {
     asm volatile("red.global.add.u64 [%0], %1;" ::"l"(a), "l"(v) : "memory");
 }
+static __device__ __forceinline__ void red_or(uint32_t *a, uint32_t v) {
+    asm volatile("red.global.or.b32 [%0], %1;" ::"l"(a), "r"(v) : "memory");
+}
 static __device__ __forceinline__ void red_max(unsigned long long *a, unsigned long long v) {
     asm volatile("red.global.max.u64 [%0], %1;" ::"l"(a), "l"(v) : "memory");
 }
@@ -89,11 +92,23 @@ static __device__ __forceinline__ void bucket_add_sums(unsigned long long *S1, u
     const unsigned long long carry = (old + lo < old) ? 1ull : 0ull;
     if (hi + carry) atomicAdd(&S2hi[idx], hi + carry);
 }
-// Add G and G^2 of one slot to bucket N*_p - 1.
+// Add G and G^2 of one slot to bucket N*_p - 1; or in two parts, the second with what the first returned.
 static __device__ __forceinline__ void bucket_add(unsigned long long *S1, unsigned long long *S2lo,
                                            unsigned long long *S2hi, int na, int bkt, int j, long long g) {
     const unsigned long long a = static_cast<unsigned long long>(g < 0 ? -g : g);
     bucket_add_sums(S1, S2lo, S2hi, na, bkt, j, g, a * a, __umul64hi(a, a));
+}
+static __device__ __forceinline__ unsigned long long bucket_add_low(unsigned long long *S1, unsigned long long *S2lo,
+                                                             int na, int bkt, int j, long long g) {
+    const size_t idx = static_cast<size_t>(bkt) * na + j;
+    atomicAdd(&S1[idx], static_cast<unsigned long long>(g));
+    return atomicAdd(&S2lo[idx], static_cast<unsigned long long>(g) * static_cast<unsigned long long>(g));
+}
+static __device__ __forceinline__ void bucket_add_high(unsigned long long *S2hi, int na, int bkt, int j, long long g,
+                                                unsigned long long old) {
+    const unsigned long long a = static_cast<unsigned long long>(g < 0 ? -g : g), lo = a * a;
+    const unsigned long long hi = __umul64hi(a, a) + (old + lo < old ? 1ull : 0ull);
+    if (hi) atomicAdd(&S2hi[static_cast<size_t>(bkt) * na + j], hi);
 }
 
 }  // namespace mcpd

@@ -58,13 +58,30 @@ enum PairStat {
 #define MCPD_HD
 #endif
 MCPD_HD inline long long pair_words(long long na, long long W) { return 2 * na + kPairStats + W; }
-// Sampling kernel: an entry is one slot's sums G [na]; a warp's scratch is `bank` entries, the list
-// of those whose pairs are done (two 32-bit words each), a statistics record per lane and, coupled,
-// sums per pair (at most 16, and one per slot of a chunk).  In 8-byte words.
-MCPD_HD inline long long warp_words(long long bank, long long na, bool coupled) {
-    return bank * na + bank + 32 * kPairStats + (coupled ? (bank < 16 ? bank : 16) * na : 0);
+// Sampling kernel: an entry is one slot's sums G [na] and `marks` words for the bit set of the clones
+// touched (mark_words); a warp's scratch is `bank` entries, the list of those whose pairs are done (two
+// 32-bit words each), a statistics record per lane and, coupled, an entry per pair (at most 16, and one
+// per slot of a chunk).  In 8-byte words.
+MCPD_HD inline long long warp_words(long long bank, long long na, long long marks, bool coupled) {
+    return (bank + (coupled ? (bank < 16 ? bank : 16) : 0)) * (na + marks) + bank + 32 * kPairStats;
 }
 #undef MCPD_HD
+// Words of an entry's marks: W 32-bit words and one for `all` (some event was not marked), or none.  A
+// slot of few steps touches few of its clones, and reading all na sums for it costs more than its steps
+// do; in small instances, or with many flips, a mark per event costs more than the reading.  Uncoupled, all
+// sums against marks: 5000 clones, 80,000 slots of 52 steps 2.4 -> 0.2 to 0.3 ms, of a sweep 5.6 -> 4; 1298
+// clones, of 52 steps 0.6 -> 0.3 to 0.5, of two sweeps 2.8 -> 2.3; 600 clones from 0.53 -> 0.37 (6 steps) to 0.66 ->
+// 0.92 (60 steps, low noise), equal at two sweeps; 333 clones mostly slower (0.89 -> 2.1 ms at worst).  Coupled:
+// 5000 clones, 9 to 800 steps 7 to 9 -> 2.2 to 3.7 ms; 2500 clones 10 to 30% less; 1298 the same.  Longer slots of
+// large instances would gain too (2500 clones, five sweeps 7.8 -> 6.7 ms).
+// steps, clones: sums over the launch's slots; a pair marks its first half sweep (mark_steps keeps out lags
+// beyond it).
+inline double mark_steps(bool coupled, int64_t B, int64_t unit, int64_t lag) {
+    return static_cast<double>(coupled ? std::max(std::max(B, unit), 2 * lag) : std::max(B, unit));
+}
+inline int32_t mark_words(bool coupled, double steps, double clones, int32_t max_na, int32_t W) {
+    return steps < (coupled ? 1.0 : 2.0) * clones && max_na >= (coupled ? 2048 : 512) ? (W + 2) / 2 : 0;
+}
 
 // Threads per block the sampling kernel is compiled for: 20 warps of 96 registers, and 16 of 128 for the
 // builds with eight row entries or a batch's descriptors.  More warps lose more to the registers they
@@ -140,7 +157,7 @@ struct KParams {
     const uint64_t *Tnu;
     const uint32_t *init_pairs;       // [n_init_pairs]
     int32_t n_init_pairs;
-    long long *pair_scratch;          // [warps][warp_words(bank, na, coupled)]
+    long long *pair_scratch;          // [warps][warp_words(bank, na, marks, coupled)]
     unsigned long long *S1;           // [nb][na]
     unsigned long long *S2lo;         // [nb][na]
     unsigned long long *S2hi;         // [nb][na]
@@ -161,6 +178,7 @@ struct KParams {
     int32_t warps;
     uint32_t smem_tables;             // bytes of staged tables at the start of shared memory
     int32_t bank, chunk;              // entries per warp; slots a warp takes at a time (<= bank)
+    int32_t marks;                    // words of marks per entry
     uint32_t rk[20];                  // Philox round keys of the seed
     int32_t nT;                       // threshold entries staged (kTSide^2, or mask-indexed)
     int32_t lag;                      // coupled lag L >= 1
@@ -208,11 +226,12 @@ struct BParams {
     int32_t n_inst, coupled, scan, max_wpp;
     int32_t lanes, max_m;             // lanes per pair (1, 8, 16, 32); largest pool count
     long long total_work, total_units;   // slots; chunks
-    long long *pair_scratch;          // [warps][warp_words(bank, max_na, coupled)], or per pair pair_words (lane groups)
+    long long *pair_scratch;          // [warps][warp_words(bank, max_na, marks, coupled)], or per pair pair_words (lane groups)
     unsigned long long *counters;
     int *error;
     int32_t max_na, max_W;
     int32_t bank;                     // entries per warp (the slots of a chunk, at most)
+    int32_t marks;                    // words of marks per entry
     int32_t ext;                      // some instance has a meeting cap or a lag > 1
     int32_t udeg;                     // every instance of the class has this uniform degree (0: mixed)
 };
@@ -244,12 +263,14 @@ inline ChunkShape chunk_shape(long long slots, long long blocks, int most, long 
 // tables: bytes staged at the start of shared memory (0 for batches); wpp: words per column;
 // P: slots of a single instance (0 = do not shape by rounds); warps: requested warps (0 = auto).
 int pairs_shape(int coupled, int scan, int udeg, bool batch, size_t tables, int wpp, size_t smem_optin,
-                long long P, int sm_count, int warps, bool ext, bool rnd, PairsShape *out);
+                long long P, int sm_count, int warps, bool ext, bool marks, PairsShape *out);
 
 // The batched sampling-kernel variants (mcpd_batch.cu): the kernel for a class, and the
 // compile-time degree a class of uniform degree udeg runs with (0: the generic build).
 using PairsKernelFn = void (*)(const KParams, const BParams);
 PairsKernelFn pick_batch(int coupled, int scan, int udeg);
+PairsKernelFn pick_marks(int coupled, int scan, bool batch, int udeg);   // the builds with marks (mcpd_marks.cu)
+PairsKernelFn pick_batch_marks(int coupled, int scan, int udeg);         // (mcpd_batch_marks.cu)
 PairsKernelFn pick_batch_degree(int udeg);                  // coupled, degrees 4, 5, 7, 8 (mcpd_batch_deg.cu)
 int batch_kernel_degree(int coupled, int ext, int udeg);
 

@@ -75,7 +75,8 @@ __global__ void philox_kernel(const uint32_t *ctr, uint32_t k0, uint32_t k1, uin
 
 using PairsFn = PairsKernelFn;
 
-PairsFn pick(int coupled, int scan, bool batch, int udeg) {
+PairsFn pick(int coupled, int scan, bool batch, int udeg, bool marks) {
+    if (marks) return pick_marks(coupled, scan, batch, udeg);
     if (batch) return pick_batch(coupled, scan, batch_kernel_degree(coupled, 0, udeg));
     if (coupled) {
         switch (udeg) {
@@ -106,9 +107,9 @@ PairsFn pick(int coupled, int scan, bool batch, int udeg) {
     }
 }
 
-int max_warps(int coupled, int scan, int udeg, bool batch) {
+int max_warps(int coupled, int scan, int udeg, bool batch, bool marks) {
     cudaFuncAttributes a{};
-    if (cudaFuncGetAttributes(&a, pick(coupled, scan, batch, udeg)) != cudaSuccess) return 16;
+    if (cudaFuncGetAttributes(&a, pick(coupled, scan, batch, udeg, marks)) != cudaSuccess) return 16;
     return a.maxThreadsPerBlock / 32;
 }
 
@@ -125,13 +126,13 @@ int pairs_max_smem(int device, size_t *bytes) {
 int launch_pairs(const KParams &kp, int grid, int block, size_t smem, void *stream) {
     if (kp.trace_rec) return launch_pairs_trace(kp, grid, block, smem, stream);
     const BParams none{};
-    pick(kp.coupled, kp.scan, false, kp.udeg)<<<grid, block, smem, static_cast<cudaStream_t>(stream)>>>(kp, none);
+    pick(kp.coupled, kp.scan, false, kp.udeg, kp.marks > 0)<<<grid, block, smem, static_cast<cudaStream_t>(stream)>>>(kp, none);
     return cudaGetLastError() == cudaSuccess ? MCPD_OK : MCPD_ECUDA;
 }
 
 int launch_batch(const BParams &bp, int grid, int block, size_t smem, void *stream) {
     const KParams none{};
-    pick(bp.coupled, bp.scan, true, bp.udeg)<<<grid, block, smem, static_cast<cudaStream_t>(stream)>>>(none, bp);
+    pick(bp.coupled, bp.scan, true, bp.udeg, bp.marks > 0)<<<grid, block, smem, static_cast<cudaStream_t>(stream)>>>(none, bp);
     return cudaGetLastError() == cudaSuccess ? MCPD_OK : MCPD_ECUDA;
 }
 
@@ -159,8 +160,8 @@ int launch_philox(const uint32_t *ctr, uint32_t k0, uint32_t k1, uint32_t *out, 
 }
 
 int pairs_shape(int coupled, int scan, int udeg, bool batch, size_t tables, int wpp, size_t smem_optin,
-                long long P, int sm_count, int warps, bool, bool, PairsShape *out) {
-    const int cap = max_warps(coupled, scan, udeg, batch);
+                long long P, int sm_count, int warps, bool, bool marks, PairsShape *out) {
+    const int cap = max_warps(coupled, scan, udeg, batch, marks);
     auto bytes = [&](int w) { return pairs_smem_bytes(tables, wpp, w); };
     auto most = [&](size_t budget) {
         int best = 0;
@@ -169,7 +170,7 @@ int pairs_shape(int coupled, int scan, int udeg, bool batch, size_t tables, int 
     };
     auto resident = [&](int w, int *per_sm) {
         *per_sm = 1;
-        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, pick(coupled, scan, batch, udeg), w * 32,
+        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, pick(coupled, scan, batch, udeg, marks), w * 32,
                                                              bytes(w)) == cudaSuccess;
     };
     // The limit of the interface: the tables and, coupled, both chains of one warp's pairs.
@@ -177,7 +178,7 @@ int pairs_shape(int coupled, int scan, int udeg, bool batch, size_t tables, int 
     int w1 = most(smem_optin);
     // The attribute is a permission shared by every launch of the kernel (the classes of a batch
     // have different sizes): allow the device's opt-in maximum.
-    if (cudaFuncSetAttribute(pick(coupled, scan, batch, udeg), cudaFuncAttributeMaxDynamicSharedMemorySize,
+    if (cudaFuncSetAttribute(pick(coupled, scan, batch, udeg, marks), cudaFuncAttributeMaxDynamicSharedMemorySize,
                              static_cast<int>(smem_optin)) != cudaSuccess)
         return MCPD_ECUDA;
     PairsShape s;

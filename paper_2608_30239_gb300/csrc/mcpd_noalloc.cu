@@ -111,9 +111,10 @@ extern "C" int mcpd_decode_noalloc(mcpd_ctx *ctx, const mcpd_design *design, con
 
     // Launch shape as the allocating path would choose it, then as many whole warps as fit.
     const size_t tables = kernel_table_bytes(t);
+    const int32_t marks = mark_words(t.coupled, mark_steps(t.coupled, t.B, t.unit, t.lag), t.na, t.na, t.W);
     PairsShape shape;
     const int src = pairs_shape(t.coupled, t.scan, t.udeg, false, tables, t.wpp, ctx->smem_optin, t.P,
-                                ctx->sm_count, 0, t.capped || t.lag > 1, !t.Tnu.empty(), &shape);
+                                ctx->sm_count, 0, t.capped || t.lag > 1, marks > 0, &shape);
     if (src == MCPD_ETOO_LARGE) return fail(ctx, src, "instance too large for the one-thread-per-pair layout");
     if (src != MCPD_OK) return fail(ctx, MCPD_ECUDA, "launch shape (cudaFuncSetAttribute / occupancy)");
     // The limit of this entry point: room for 32 pairs' accumulators of pair_words and a column each.
@@ -129,12 +130,12 @@ extern "C" int mcpd_decode_noalloc(mcpd_ctx *ctx, const mcpd_design *design, con
     for (bool first = true;; first = false) {
         chunk = static_cast<int>(std::min<long long>(32, 4 * up(t.P, 4ll * grid * warps)));
         if (first) warps = static_cast<int>(std::min<long long>(warps, up(t.P, static_cast<long long>(grid) * chunk)));
-        if (static_cast<size_t>(grid) * warps * warp_words(chunk, t.na, t.coupled) * 8 <= room || (grid == 1 && warps == 1)) break;
+        if (static_cast<size_t>(grid) * warps * warp_words(chunk, t.na, marks, t.coupled) * 8 <= room || (grid == 1 && warps == 1)) break;
         if (warps > 1) --warps; else --grid;
     }
     const size_t smem = pairs_smem_bytes(tables, t.wpp, warps);
     const size_t all_warps = static_cast<size_t>(grid) * warps;
-    const size_t o_pair = take(all_warps * static_cast<size_t>(warp_words(chunk, t.na, t.coupled)) * 8);
+    const size_t o_pair = take(all_warps * static_cast<size_t>(warp_words(chunk, t.na, marks, t.coupled)) * 8);
     if (off > kNoAllocScratchBytes) return fail(ctx, MCPD_ETOO_LARGE, "no-alloc scratch layout overflow");
 
     unsigned char *b = static_cast<unsigned char *>(base);
@@ -174,6 +175,7 @@ extern "C" int mcpd_decode_noalloc(mcpd_ctx *ctx, const mcpd_design *design, con
     kp.smem_tables = static_cast<uint32_t>(tables);
     kp.nT = static_cast<int32_t>(kernel_T(t).size());
     kp.bank = chunk;
+    kp.marks = marks;
     kp.chunk = chunk;
     if (launch_pairs(kp, grid, warps * 32, smem, s) != MCPD_OK)
         return fail(ctx, MCPD_ECUDA, std::string("pairs kernel launch: ") + cudaGetErrorString(cudaGetLastError()));

@@ -37,7 +37,7 @@ namespace {
 // Why apart: in one loop for both, the few unmet lanes of a warp (4.8% of lane-steps, at least one
 // in 79% of warp-steps) made every step pay for Y, and the replications of a warp ended one by one.
 // Running X's first tau steps twice costs tau / l (5% there).
-template <bool COUPLED, bool SYSTEMATIC, bool BATCH, int DEG, bool TRACE = false>
+template <bool COUPLED, bool SYSTEMATIC, bool BATCH, int DEG, bool TRACE = false, bool MARKS = false>
 __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(const KParams p, const BParams bp) {
     extern __shared__ __align__(16) unsigned char smem[];
     constexpr unsigned FULL = 0xFFFFFFFFu;
@@ -69,14 +69,17 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
     if constexpr (!BATCH) st[p.dummy_word_index * 32] = p.dummy_word;
     __syncthreads();
 
-    // This warp's scratch (see warp_words): `bank` entries (a slot's sums), a list of the entries
-    // whose pairs are done, a statistics record per lane, and sums per pair.
+    // This warp's scratch (see warp_words): `bank` entries (a slot's sums, and marks of the clones
+    // touched), a list of the entries whose pairs are done, a statistics record per lane, and an entry
+    // per pair.
     const int stride_na = BATCH ? bp.max_na : p.na;
-    const int bank = BATCH ? bp.bank : p.bank;
+    const int bank = BATCH ? bp.bank : p.bank, marks = MARKS ? (BATCH ? bp.marks : p.marks) : 0;
     long long *const wbase = (BATCH ? bp.pair_scratch : p.pair_scratch) +
                              static_cast<size_t>(blockIdx.x * nwarps + warp) *
-                                 static_cast<size_t>(warp_words(bank, stride_na, COUPLED));
-    const size_t ew = static_cast<size_t>(stride_na);
+                                 static_cast<size_t>(warp_words(bank, stride_na, marks, COUPLED));
+    const size_t ew = static_cast<size_t>(stride_na) + static_cast<size_t>(marks);
+    // Word q of the marks of an entry; word W: events that were not marked.
+    auto mark = [&](long long *entry, uint32_t q) { return reinterpret_cast<uint32_t *>(entry + stride_na) + q; };
     auto list = [&]() { return reinterpret_cast<uint32_t *>(wbase + bank * ew); };
     auto pst = [&]() {
         return reinterpret_cast<unsigned long long *>(wbase + bank * ew + bank + lane * kPairStats);
@@ -95,6 +98,9 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
     const unsigned long long *gAlias = nullptr, *gT = nullptr;
     int na = 0, deg = 0;
     uint32_t W = 0, ell = 0, instance = 0, k0 = 0, k1 = 0, dummy_entry = 0, ws0 = 0, wcap = 0;
+    // A pair marks its events up to this step; one that goes on leaves its slot to be read whole, so that a
+    // long one does not pay for a mark per event as well.
+    auto marked_steps = [&]() { return static_cast<uint32_t>(na) >> 1; };
 #define MCPD_FIELD(name, batch_expr, single_expr) \
     auto name = [&]() { if constexpr (BATCH) return batch_expr; else return single_expr; }
     MCPD_FIELD(v_B, static_cast<uint32_t>(__ldg(&desc->B)), static_cast<uint32_t>(p.B));
@@ -305,6 +311,7 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
         for (uint32_t q = lane, e = v_wpp(); q < e; q += 32) {
             if (q < W && w_s) {
                 uint32_t m = st_s[q * 32];
+                if (MARKS && m) red_or(mark(sum_s, q), m);
                 while (m) {
                     const int b = __ffs(m) - 1;
                     m &= m - 1;
@@ -324,26 +331,23 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
                 p.trace_G[(static_cast<long long>(slot) / p.trace_stride) * na + j] = g;
         }
     };
-    // Add entry `idx` to bucket n - 1 (n = 0: the slot is dropped) and zero it, by the whole warp:
-    // coalesced reads of all its sums, four in flight a lane.  (Marking the touched clones with a
-    // reduction per flip, to read only those here, cost every flip more than reading na sums once
-    // per slot.)
+    // Add sum g of clone j of entry `idx` to bucket n - 1 (n = 0: the slot is dropped) and zero it.
+    auto move = [&](uint32_t idx, uint32_t n, int j, long long g) {
+        if (g == 0) return;
+        wbase[static_cast<size_t>(idx) * ew + j] = 0;
+        if (!n) return;
+        bucket_add(v_S1(), v_S2lo(), v_S2hi(), na, static_cast<int>(n) - 1, j, g);
+        trace_sum(idx, j, g);
+    };
+    // All sums of entry `idx`, by the whole warp: coalesced reads, four in flight a lane.
     auto flush = [&](uint32_t idx, uint32_t n) {
-        long long *const from = wbase + static_cast<size_t>(idx) * ew;
+        const long long *const from = wbase + static_cast<size_t>(idx) * ew;
         for (int j0 = lane; j0 < na; j0 += 128) {
             long long g[4];
 #pragma unroll
             for (int u = 0; u < 4; ++u) g[u] = j0 + 32 * u < na ? __ldcg(from + j0 + 32 * u) : 0;
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                if (g[u] == 0) continue;
-                const int j = j0 + 32 * u;
-                from[j] = 0;
-                if (n) {
-                    bucket_add(v_S1(), v_S2lo(), v_S2hi(), na, static_cast<int>(n) - 1, j, g[u]);
-                    trace_sum(idx, j, g[u]);
-                }
-            }
+            for (int u = 0; u < 4; ++u) move(idx, n, j0 + 32 * u, g[u]);
         }
         if (lane == 0 && n) atomicAdd(&v_bcount()[n - 1], 1ull);
     };
@@ -373,6 +377,71 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
             if (lo | hi) bucket_add_sums(v_S1(), v_S2lo(), v_S2hi(), na, static_cast<int>(n) - 1, j, s1, lo, hi);
         }
         if (lane == 0) atomicAdd(&v_bcount()[n - 1], static_cast<unsigned long long>(cnt));
+    };
+    // The marked sums of the list's entries, eight entries at a time: a lane takes the next marked clone of
+    // each of four, so that four loads, and then four additions, are in flight (one by one, 80,000 slots of 4
+    // steps of 5000 clones took 0.18 to 0.38 ms); an entry with events that were not marked is read whole.
+    auto flush_marked = [&](uint32_t entries_done, uint32_t reps_each) {
+        constexpr int G = 8;
+        for (uint32_t at = 0; at < entries_done; at += G) {
+            const bool mine = lane < G && at + lane < entries_done;
+            const uint32_t my_idx = !mine ? 0u : COUPLED ? __ldcg(list() + 2 * (at + lane)) : at + lane;
+            const uint32_t my_n = !mine ? 0u : COUPLED ? __ldcg(list() + 2 * (at + lane) + 1) : reps_each;
+            bool whole = false;
+            if constexpr (COUPLED) {
+                uint32_t *const my_all = mark(wbase + my_idx * ew, W);
+                whole = mine && __ldcg(my_all) != 0u;
+                if (whole) *my_all = 0u;
+            }
+            const unsigned all = __ballot_sync(FULL, whole), here = __ballot_sync(FULL, mine);
+            uint32_t idx[G], n[G];
+#pragma unroll
+            for (int u = 0; u < G; ++u) {
+                idx[u] = __shfl_sync(FULL, my_idx, u);
+                n[u] = __shfl_sync(FULL, my_n, u);
+            }
+            for (uint32_t q = lane; q < W; q += 32) {
+                uint32_t m[G];
+#pragma unroll
+                for (int u = 0; u < G; ++u) m[u] = (here >> u) & 1u ? __ldcg(mark(wbase + idx[u] * ew, q)) : 0u;
+#pragma unroll
+                for (int u = 0; u < G; ++u) {
+                    if (m[u]) *mark(wbase + idx[u] * ew, q) = 0u;
+                    if ((all >> u) & 1u) m[u] = 0u;
+                }
+#pragma unroll
+                for (int h = 0; h < G; h += 4)
+                    while (m[h] | m[h + 1] | m[h + 2] | m[h + 3]) {
+                        long long g[4];
+                        unsigned long long old[4];
+                        uint32_t j[4];
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            j[u] = q * 32u + static_cast<uint32_t>(__ffs(m[h + u])) - 1u;
+                            g[u] = m[h + u] ? __ldcg(wbase + idx[h + u] * ew + j[u]) : 0;
+                            m[h + u] &= m[h + u] - 1u;
+                        }
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            if (g[u] == 0) continue;
+                            wbase[idx[h + u] * ew + j[u]] = 0;
+                            if (!n[h + u]) continue;
+                            old[u] = bucket_add_low(v_S1(), v_S2lo(), na, static_cast<int>(n[h + u]) - 1, static_cast<int>(j[u]), g[u]);
+                            trace_sum(idx[h + u], static_cast<int>(j[u]), g[u]);
+                        }
+#pragma unroll
+                        for (int u = 0; u < 4; ++u)
+                            if (g[u] && n[h + u])
+                                bucket_add_high(v_S2hi(), na, static_cast<int>(n[h + u]) - 1, static_cast<int>(j[u]), g[u], old[u]);
+                    }
+            }
+            __syncwarp();
+            if (COUPLED && mine && !whole && my_n) atomicAdd(&v_bcount()[my_n - 1], 1ull);
+#pragma unroll
+            for (int u = 0; u < G; ++u)
+                if ((all >> u) & 1u) flush(idx[u], n[u]);
+        }
+        if (!COUPLED && lane == 0) atomicAdd(&v_bcount()[reps_each - 1], static_cast<unsigned long long>(entries_done));
     };
     auto record_slot = [&](uint32_t nstar, long long cost, uint32_t reps) {
         if constexpr (!BATCH) {
@@ -530,6 +599,7 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
                                               static_cast<long long>(static_cast<unsigned long long>(single ? 0u : u - m) * wcap);
                                 if (lag != 1u && !single) w = lag_prefix(u, ws0, ell, lag);
                                 red_add(sum + s.I, (s.z != 0) != (role == 3) ? w : -w);
+                                if (MARKS && (single || t < marked_steps())) red_or(mark(sum, s.q), 1u << (s.I & 31));
                                 events = true;
                             }
                         }
@@ -591,6 +661,7 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
                                         const uint32_t xw = st[q * 32];
                                         uint32_t dm = xw ^ st[q * 32 + 16];
                                         if (!dm) continue;
+                                        if (MARKS) red_or(mark(entry(), q), dm);
                                         while (dm) {
                                             const int b = __ffs(dm) - 1;
                                             dm &= dm - 1;
@@ -648,7 +719,25 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
                                 const bool keep_s = __shfl_sync(FULL, keep ? 1 : 0, src) != 0;
                                 long long *const to = wbase + static_cast<size_t>(__shfl_sync(FULL, slot_local, src) - first) * ew;
                                 long long *const from = pair_sums(src);
-                                for (int j0 = lane; j0 < na; j0 += 128) {
+                                bool all = true;
+                                if constexpr (MARKS) {
+                                    all = __shfl_sync(FULL, t, src) > marked_steps();
+                                    for (uint32_t q = lane; q < W; q += 32) {
+                                        uint32_t b = __ldcg(mark(from, q));
+                                        if (!b) continue;
+                                        *mark(from, q) = 0u;
+                                        if (keep_s) red_or(mark(to, q), b);
+                                        while (!all && b) {
+                                            const uint32_t j = q * 32 + __ffs(b) - 1;
+                                            b &= b - 1;
+                                            const long long g = __ldcg(from + j);
+                                            from[j] = 0;
+                                            if (keep_s) red_add(to + j, g);
+                                        }
+                                    }
+                                    if (all && keep_s && lane == 0) red_or(mark(to, W), 1u);
+                                }
+                                for (int j0 = all ? lane : na; j0 < na; j0 += 128) {
                                     long long g[4];
 #pragma unroll
                                     for (int u = 0; u < 4; ++u) g[u] = j0 + 32 * u < na ? __ldcg(from + j0 + 32 * u) : 0;
@@ -797,7 +886,10 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
                         if (f) {
                             apply(s);
                             const uint32_t w = wstep(time);
-                            if (w) red_add(sum + s.I, s.z ? static_cast<long long>(w) : -static_cast<long long>(w));
+                            if (w) {
+                                red_add(sum + s.I, s.z ? static_cast<long long>(w) : -static_cast<long long>(w));
+                                if (MARKS) red_or(mark(sum, s.q), 1u << (s.I & 31));
+                            }
                         }
                     }
                 };
@@ -831,6 +923,7 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
                     if (xw) {
                         st[q * 32] = 0u;
                         uint32_t m = w ? xw : 0u;
+                        if (MARKS && m) red_or(mark(sum, q), m);
                         while (m) {
                             const int b = __ffs(m) - 1;
                             m &= m - 1;
@@ -855,7 +948,8 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
         // before they are read, and the zeros before the next chunk reduces into them.
         __threadfence();
         __syncwarp();
-        if constexpr (!COUPLED) flush_same(reps_each);
+        if constexpr (MARKS) flush_marked(ready, reps_each);
+        else if constexpr (!COUPLED) flush_same(reps_each);
         else for (uint32_t at = 0; at < ready; ++at) flush(__ldcg(list() + 2 * at), __ldcg(list() + 2 * at + 1));
         __threadfence();
         __syncwarp();

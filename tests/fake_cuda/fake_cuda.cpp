@@ -20,7 +20,7 @@ int g_device = 0;
 cudaError_t g_last = cudaSuccess;
 std::map<char *, size_t> g_blocks;
 // One launch: lanes, grid, warps per block, bank, total chunks, instances, words of its scratch that
-// are allocated; then per instance: slots, first chunk, chunks, clones.
+// are allocated, words of marks per entry; then per instance: slots, first chunk, chunks, clones.
 std::vector<long long> g_log;
 
 size_t room_at(const void *p) {
@@ -123,7 +123,7 @@ static int log_launch(const BParams &bp, int grid, int block) {
     const size_t words = room_at(bp.pair_scratch) / 8;
     for (long long v : {static_cast<long long>(bp.lanes), static_cast<long long>(grid), static_cast<long long>(block / 32),
                         static_cast<long long>(bp.bank), bp.total_units, static_cast<long long>(bp.n_inst),
-                        static_cast<long long>(words)})
+                        static_cast<long long>(words), static_cast<long long>(bp.marks)})
         g_log.push_back(v);
     for (int i = 0; i < bp.n_inst; ++i)
         for (long long v : {bp.insts[i].P, bp.insts[i].unit_begin, bp.insts[i].units, static_cast<long long>(bp.insts[i].na)})
@@ -135,7 +135,7 @@ int launch_group(const BParams &bp, int grid, int block, size_t, void *) { retur
 int launch_pairs(const KParams &kp, int grid, int block, size_t, void *) {
     if (cudaGetLastError() != cudaSuccess) return MCPD_ECUDA;
     for (long long v : {0ll, static_cast<long long>(grid), static_cast<long long>(block / 32), static_cast<long long>(kp.bank),
-                        static_cast<long long>(kp.chunk), 1ll, static_cast<long long>(room_at(kp.pair_scratch) / 8), kp.P, 0ll, 0ll,
+                        static_cast<long long>(kp.chunk), 1ll, static_cast<long long>(room_at(kp.pair_scratch) / 8), static_cast<long long>(kp.marks), kp.P, 0ll, 0ll,
                         static_cast<long long>(kp.na)})
         g_log.push_back(v);
     return MCPD_OK;

@@ -41,9 +41,9 @@ class Host:
         self.lib.fake_log(v.ctypes.data, n)
         got, at = [], 0
         while at < n:
-            d = dict(zip(("lanes", "grid", "warps", "bank", "units", "n_inst", "words"), v[at:at + 7].tolist()))
-            d["inst"] = v[at + 7:at + 7 + 4 * d["n_inst"]].reshape(-1, 4)       # slots, first chunk, chunks, clones
-            at += 7 + 4 * d["n_inst"]
+            d = dict(zip(("lanes", "grid", "warps", "bank", "units", "n_inst", "words", "marks"), v[at:at + 8].tolist()))
+            d["inst"] = v[at + 8:at + 8 + 4 * d["n_inst"]].reshape(-1, 4)       # slots, first chunk, chunks, clones
+            at += 8 + 4 * d["n_inst"]
             got.append(d)
         return got
 
@@ -63,8 +63,8 @@ def host(tmp_path_factory):
     mcpd._lib, build.LIB = kept
 
 
-def warp_words(bank, na):
-    return bank * na + bank + 32 * PAIR_STATS + min(bank, 16) * na          # coupled
+def warp_words(bank, na, marks=0, coupled=True):
+    return (bank + coupled * min(bank, 16)) * (na + marks) + bank + 32 * PAIR_STATS
 
 
 def check(launches, slots):
@@ -72,7 +72,7 @@ def check(launches, slots):
     total = 0
     for d in launches:
         na = int(d["inst"][:, 3].max())
-        assert d["grid"] * d["warps"] * warp_words(d["bank"], na) <= d["words"]
+        assert d["grid"] * d["warps"] * warp_words(d["bank"], na, d["marks"]) <= d["words"]
         at = 0
         for P, begin, units, _ in d["inst"].tolist():
             assert begin == at
@@ -173,7 +173,7 @@ def test_failed_shape_change_keeps_the_shape(host):
     its launches find no error left over."""
     insts = [synth.make_instance(4000, 100, 4, 2, 0.05, 0.1, 0.003, i, 50 + i) for i in range(8)]
     slots = 8 * 2432
-    b = mcpd.Batch(host.ctx, insts, [dict(slots=2432, horizon=4000, seed=i, instance_id=i) for i in range(8)], classes=2)
+    b = mcpd.Batch(host.ctx, insts, [dict(slots=2432, horizon=12000, seed=i, instance_id=i) for i in range(8)], classes=2)
     rc, got = host.run(b)
     assert rc == 0
     words = [d["words"] for d in got]
@@ -252,3 +252,30 @@ def test_plan_in_less_memory(host, part):
     finally:
         host.lib.fake_budget(1 << 40)
     assert host.lib.fake_live() == base
+
+
+@pytest.mark.parametrize("n,kw,marks", [
+    (2048, dict(k=0, ell=30, horizon=2047), 33), (2048, dict(k=0, ell=30, horizon=2048), 0), (2047, dict(k=0, ell=30, horizon=90), 0),
+    (2048, dict(k=0, ell=30, horizon=90, lag=1023), 33), (2048, dict(k=0, ell=30, horizon=90, lag=1024), 0),
+    (512, dict(coupled=False, burn=5, length=20, horizon=1023), 9), (512, dict(coupled=False, burn=5, length=20, horizon=1024), 0),
+    (511, dict(coupled=False, burn=5, length=20, horizon=0), 0), (512, dict(coupled=False, burn=5, length=2000, horizon=0), 0),
+    (2048, dict(k=0, ell=30, horizon=90, trace_stride=1, trace_steps=5), 0)])
+def test_marks_rule(host, n, kw, marks):
+    """Words of marks (W bit words, two to a word, and one 32-bit word more) where slots are short for their clones, and
+    scratch for them."""
+    inst = synth.make_instance(n, n // 13, 4, 2, 0.05, 0.1, 2 / n, 1, 2)
+    out = np.zeros(n)
+    plan = mcpd.Plan(host.ctx, inst, slots=500, seed=3, **kw)
+    host.lib.fake_clear_log()
+    assert mcpd.lib().mcpd_run_async(host.ctx.h, plan.h, out.ctypes.data, out.ctypes.data) == 0
+    d, = host.launches()
+    assert d["marks"] == marks
+    assert d["grid"] * d["warps"] * warp_words(d["bank"], n, marks, kw.get("coupled", True)) <= d["words"]
+    plan.close()
+    if "trace_steps" not in kw:
+        b = mcpd.Batch(host.ctx, [inst, inst], dict(slots=500, seed=3, **kw))
+        rc, got = host.run(b)
+        assert rc == 0 and [g["marks"] for g in got] == [marks]
+        if kw.get("coupled", True):
+            check(got, 1000)
+        b.close()
