@@ -216,9 +216,12 @@ int mcpd_ctx_create(int device, void *cuda_stream, mcpd_ctx **out) {
 void mcpd_ctx_destroy(mcpd_ctx *ctx) {
     if (!ctx) return;
     if (ctx->stage_bytes) {
-        cudaSetDevice(ctx->device);
+        int current = ctx->device;         // the calling thread keeps its device
+        cudaGetDevice(&current);
+        if (current != ctx->device) cudaSetDevice(ctx->device);
         cudaFreeHost(ctx->stage_host);
         cudaFree(ctx->stage_dev);
+        if (current != ctx->device) cudaSetDevice(current);
     }
     delete ctx;
 }

@@ -42,6 +42,11 @@ long long fake_log(long long *out, long long cap) {
     for (long long i = 0; i < std::min(n, cap); ++i) out[i] = g_log[static_cast<size_t>(i)];
     return n;
 }
+void fake_stage(mcpd_ctx *ctx) {       // as a call of mcpd_features_batch leaves it
+    ctx->stage_host = std::malloc(64);
+    cudaMalloc(&ctx->stage_dev, 64);
+    ctx->stage_bytes = 64;
+}
 void fake_clear_log() { g_log.clear(); }
 
 cudaError_t cudaMalloc(void **p, size_t bytes) {

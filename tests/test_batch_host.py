@@ -21,7 +21,7 @@ class Host:
         self.lib = lib
         for name, res, args in (("fake_budget", None, [C.c_int64]), ("fake_allocs", None, [C.c_int64]),
                                 ("fake_live", C.c_int64, []),
-                                ("fake_device", C.c_int, [C.c_int]), ("fake_clear_log", None, []),
+                                ("fake_device", C.c_int, [C.c_int]), ("fake_stage", None, [C.c_void_p]), ("fake_clear_log", None, []),
                                 ("fake_log", C.c_int64, [C.c_void_p, C.c_int64])):
             f = getattr(lib, name)
             f.restype, f.argtypes = res, args
@@ -279,3 +279,17 @@ def test_marks_rule(host, n, kw, marks):
         if kw.get("coupled", True):
             check(got, 1000)
         b.close()
+
+
+@pytest.mark.parametrize("staged", [False, True])
+def test_destroying_a_context_keeps_the_current_device(host, staged):
+    live = host.lib.fake_live()
+    c = mcpd.Context(0, stream=1)
+    if staged:
+        host.lib.fake_stage(c.h)
+    host.lib.fake_device(1)
+    try:
+        c.close()
+        assert host.lib.fake_device(-1) == 1 and host.lib.fake_live() == live
+    finally:
+        host.lib.fake_device(0)
