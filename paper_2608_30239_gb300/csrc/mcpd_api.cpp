@@ -259,7 +259,7 @@ int mcpd_plan_create(mcpd_ctx *ctx, const mcpd_design *design, const uint8_t *y,
                            ctx->sm_count, 0, t.capped || t.lag > 1, marks > 0, &shape);
     if (rc != MCPD_OK) {
         delete pl;
-        return set_err(ctx, rc, rc == MCPD_ETOO_LARGE ? "instance too large for the one-thread-per-pair layout"
+        return set_err(ctx, rc, rc == MCPD_ETOO_LARGE ? "instance too large: its tables and one warp's pairs exceed shared memory"
                                                       : "launch shape (cudaFuncSetAttribute / occupancy)");
     }
     const int warps = shape.warps;

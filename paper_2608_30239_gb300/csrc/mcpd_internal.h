@@ -249,9 +249,9 @@ inline size_t pairs_smem_bytes(size_t tables, int wpp, int warps) {
 // slots a warp takes at a time (a chunk).  All of a warp's share at once (in equal parts if a bank
 // cannot hold it): a chunk's single runs are dealt to the lanes one by one, so any number of slots fills
 // them, and its pairs fill a warp the better the more there are.  All warps once the slots give each
-// 16 pairs; below that at most kSpreadWarps per block: 16384 slots with a lag of one sweep, whose time is
-// its pairs', took 37 and 28 ms (two seeds) on 23 warps of 5 slots, 31.5 and 21.7 ms on 12 of 9, 33 and
-// 23 ms on 8 of 14.
+// 16 pairs; below that at most kSpreadWarps per block, since the time of few slots is their pairs':
+// 16384 slots with a lag of one sweep take 14.5, 14.5, 15.8 and 17.9 ms on at most 8, 12, 16 and 20 warps
+// (4096 slots 10.2, 11.7, 13.2, 15.6; without the lag 16384 slots 5.7, 5.3, 5.3, 5.6; 1298 x 97, high noise).
 constexpr int kSpreadWarps = 12;
 struct ChunkShape { int warps, chunk; };
 inline ChunkShape chunk_shape(long long slots, long long blocks, int most, long long bank) {
@@ -261,7 +261,8 @@ inline ChunkShape chunk_shape(long long slots, long long blocks, int most, long 
     return {static_cast<int>(w), static_cast<int>(up(share, up(share, bank)))};
 }
 // tables: bytes staged at the start of shared memory (0 for batches); wpp: words per column;
-// P: slots of a single instance (0 = do not shape by rounds); warps: requested warps (0 = auto).
+// P: slots of a single instance (0: as many warps as fit); warps: requested warps (0 = auto); marks:
+// the builds with marks.
 int pairs_shape(int coupled, int scan, int udeg, bool batch, size_t tables, int wpp, size_t smem_optin,
                 long long P, int sm_count, int warps, bool ext, bool marks, PairsShape *out);
 

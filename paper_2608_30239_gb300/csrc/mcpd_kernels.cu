@@ -5,11 +5,11 @@
 // lanes to a pair, and then its single chains, a lane each, under the fixed horizon B with slot
 // refill (Algorithm 4).  Per lane, shared memory holds one chain's clone bit set and its
 // per-pool positive counts (one byte each), laid out word-interleaved over the warp's 32 lanes so
-// that the per-step loads of different lanes never share a bank.  The clone->pool rows, the alias table of the scan weights and the acceptance
-// thresholds are staged once per block.  The hot loop is integer-only: a Philox4x32-10 block
+// that the per-step loads of different lanes never share a bank.  The clone->pool rows, the alias
+// table of the scan weights and the acceptance thresholds are staged once per block.  The hot loop is integer-only: a Philox4x32-10 block
 // feeds two steps, the site comes from the alias table, the full conditional from a table lookup
 // indexed by (n+, n-), and the update from a 64-bit integer comparison.  The estimator
-// H_{k:l} is accumulated exactly in integers, only when a site flips (see wprefix below), and
+// H_{k:l} is accumulated exactly in integers, only when a site flips (see the head of mcpd_pairs.cuh), and
 // slot sums go to N*_p buckets with 64/128-bit integer atomics, so the result does not depend on
 // the schedule.
 #include <cuda_runtime.h>

@@ -115,7 +115,7 @@ extern "C" int mcpd_decode_noalloc(mcpd_ctx *ctx, const mcpd_design *design, con
     PairsShape shape;
     const int src = pairs_shape(t.coupled, t.scan, t.udeg, false, tables, t.wpp, ctx->smem_optin, t.P,
                                 ctx->sm_count, 0, t.capped || t.lag > 1, marks > 0, &shape);
-    if (src == MCPD_ETOO_LARGE) return fail(ctx, src, "instance too large for the one-thread-per-pair layout");
+    if (src == MCPD_ETOO_LARGE) return fail(ctx, src, "instance too large: its tables and one warp's pairs exceed shared memory");
     if (src != MCPD_OK) return fail(ctx, MCPD_ECUDA, "launch shape (cudaFuncSetAttribute / occupancy)");
     // The limit of this entry point: room for 32 pairs' accumulators of pair_words and a column each.
     if (fixed + 2 * 256 > kNoAllocScratchBytes)

@@ -354,7 +354,8 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
     // All sums of entries 0 .. cnt - 1, whose slots all retained n replications (uncoupled chains): a lane
     // adds a clone's sums over the slots and brings the totals to the bucket.  (Slot by slot, every slot's
     // three atomics per clone met all other warps' on the bucket: 4.7 million chains of 32 steps on 64 clones
-    // took 13.5 ms against 1.7, 0.9 million of one sweep on 333 clones 2.6 against 1.8.)
+    // took 13.5 ms against 1.7, 0.9 million of one sweep on 333 clones 2.6 against 1.8.)  For fewer than four
+    // slots, whose loads in flight are too few: 81 slots of 2424 clones 481 us this way, 458 one by one.
     auto flush_same = [&](uint32_t n) {
         for (int j = lane; j < na; j += 32) {
             long long s1 = 0;
@@ -949,7 +950,8 @@ __global__ void __launch_bounds__(pairs_threads(DEG, BATCH), 1) pairs_kernel(con
         __threadfence();
         __syncwarp();
         if constexpr (MARKS) flush_marked(ready, reps_each);
-        else if constexpr (!COUPLED) flush_same(reps_each);
+        else if (!COUPLED && cnt >= 4) flush_same(reps_each);
+        else if constexpr (!COUPLED) for (uint32_t at = 0; at < cnt; ++at) flush(at, reps_each);
         else for (uint32_t at = 0; at < ready; ++at) flush(__ldcg(list() + 2 * at), __ldcg(list() + 2 * at + 1));
         __threadfence();
         __syncwarp();

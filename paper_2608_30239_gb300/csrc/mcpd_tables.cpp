@@ -205,10 +205,9 @@ int build_tables(const mcpd_design *d, const uint8_t *y, const mcpd_params *prm,
             if (t.Tnu[a] || (a + 1 < na && t.Tnu[a + 1])) t.init_pairs.push_back(static_cast<uint32_t>(a));
     }
 
-    // Shared-memory layout of one pair (the X chain): W words of bits, then one count byte per
-    // pool, the padding pool m last.  Word w of a pair lives at word (w * 32 + lane) of its warp's
-    // region, so the byte of pool j sits at (W + j / 4) * 128 + j % 4 from the lane's base.  The Y
-    // chain uses the same layout, contiguous, in global memory while the pair has not met.
+    // Shared-memory layout of one chain: W words of bits, then one count byte per pool, the padding
+    // pool m last.  Word w of a lane's chain lives at word (w * 32 + lane) of its warp's region, so
+    // the byte of pool j sits at (W + j / 4) * 128 + j % 4 from the lane's base.
     t.W = (na + 31) / 32;
     t.Mp = (m + 1 + 3) / 4;
     t.wpp = t.W + t.Mp;

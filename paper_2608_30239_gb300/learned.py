@@ -250,7 +250,7 @@ def time_to_se(ctx, inst, target=0.005, sweeps=29.4, seed=7, weights=None, init=
     creation through the copy of the SEs that met the target (`wall_ms`), the slots used, the final
     largest SE, whether it met the target, and the path [(slots so far, max SE, kernel ms so far)].
     The plan is shaped for `plan_slots` slots (the launch shape of the bench's decode); every range
-    keeps its grid and trims its warps per block to whole rounds of the range."""
+    keeps its grid, with the warps per block and the slots per warp fitted to the range."""
     import torch
     t0 = time.perf_counter()
     kw = dict(slots=plan_slots, horizon=int(sweeps * inst.n), seed=seed)
