@@ -1,7 +1,8 @@
 // The persistent sampling kernel (template): a warp runs a chunk of slots, each slot's pairs to
 // their meetings first and its single chains after (Algorithms 3 and 4).  Included by the
 // translation units that instantiate it: mcpd_kernels.cu and mcpd_batch*.cu (the production
-// variants) and mcpd_trace.cu (the variants that also record per-replication trajectories).
+// variants), mcpd_marks.cu and mcpd_batch_marks.cu (MARKS: slots of few steps, see mark_words) and
+// mcpd_trace.cu (TRACE: the variants that also record per-replication trajectories).
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
